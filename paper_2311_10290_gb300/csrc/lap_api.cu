@@ -44,6 +44,7 @@ void free_all(lap_graph *g)
     cudaFree(g->d_row_ptr);
     cudaFree(g->d_col);
     cudaFree(g->d_rowinfo);
+    cudaFree(g->d_arcs);
     cudaFree(g->d_hops);
     cudaFree(g->d_rep1);
     cudaFree(g->d_cnt2);
@@ -164,6 +165,7 @@ int choose_kernel(const lap_graph *g, uint64_t n_samples = 0)
 lap_status ensure_workspace(lap_graph *g, int kernel)
 {
     const uint64_t per_slot = slot_bytes_of(g, kernel);
+    g->blk_clean = 0;
     if (!g->ws) {
         size_t free_b = 0, total_b = 0;
         LAP_CUDA(g, cudaMemGetInfo(&free_b, &total_b));
@@ -237,6 +239,49 @@ lap_status launch(lap_graph *g, LapSampleLaunch &p, int kernel)
         g->sticky = LAP_ERR_CUDA;
         return fail(g, LAP_ERR_CUDA, buf);
     }
+    return LAP_OK;
+}
+
+constexpr int32_t kBlockMinNodes = 2048;
+
+// The block kernel (sampler_block.cu) takes automatic calls and kernel 3 with
+// the automatic number of walkers, where it applies: `pl` is the launch then.
+bool choose_block(const lap_graph *g, uint64_t n_samples, LapBlockPlan *pl)
+{
+    if (g->walkers || g->compact_disabled || !g->ws || (g->kernel_opt == 0 && g->n < kBlockMinNodes)) return false;
+    if (g->kernel_opt != 0 && g->kernel_opt != LAP_KERNEL_GROUP) return false;
+    return lap_block_plan(g->n, n_samples, g->slots_opt, g->ws_bytes, g->num_sms, g->paths_opt != 0, g->cv1 || g->cv2,
+                          g->d_arcs != nullptr, pl);
+}
+
+lap_status launch_block(lap_graph *g, LapSampleLaunch &p, LapBlockPlan &pl)
+{
+    // The tagged words are zeroed when the workspace last held something else
+    // there, and when the tags (31 bits) run out.
+    if (pl.words_bytes > g->blk_clean || (uint64_t)g->tag_next + p.count + 1ull >= (1ull << 31)) {
+        LAP_CUDA(g, cudaMemsetAsync(g->ws, 0, pl.words_bytes, g->stream));
+        g->tag_next = 0;
+    }
+    g->blk_clean = pl.words_bytes;
+    g->last_kernel = LAP_KERNEL_GROUP;
+    g->ws_zeroed = false;
+    uint8_t *ws = reinterpret_cast<uint8_t *>(g->ws);
+    p.slots = pl.slots;
+    pl.b.arcs = g->d_arcs;
+    if (g->d_arcs) lap_pack_bits(g->n, g->arcs, &pl.b.bw, &pl.b.bo);
+    pl.b.tag_base = g->tag_next;
+    pl.b.words = reinterpret_cast<unsigned long long *>(ws);
+    pl.b.path_words = reinterpret_cast<unsigned long long *>(ws + pl.path_offset);
+    pl.b.stacks = reinterpret_cast<uint2 *>(ws + pl.stack_offset);
+    pl.b.sweep = reinterpret_cast<uint32_t *>(ws + pl.sweep_offset);
+    pl.b.early = reinterpret_cast<uint32_t *>(ws + pl.early_offset);
+    pl.b.early_stacks = pl.b.early + (uint64_t)pl.b.early_entries * pl.b.early_count;
+    pl.b.early_pops = pl.b.early_stacks + (uint64_t)pl.b.early_cap * pl.b.early_count;
+    g->tag_next += p.count;
+    LAP_CUDA(g, cudaMemsetAsync(&g->d_acc->claim, 0, sizeof(unsigned int), g->stream));
+    LAP_CUDA(g, cudaMemsetAsync(&g->d_acc->walk_claim, 0, sizeof(unsigned int), g->stream));
+    const cudaError_t e = lap_launch_sample_block(p, pl, g->stream);
+    if (e != cudaSuccess) return cuda_fail(g, e, "sampler launch (block kernel)");
     return LAP_OK;
 }
 
@@ -375,6 +420,16 @@ lap_status lap_graph_create(int32_t n, const int32_t *row_ptr, const int32_t *co
         return bad;
     }
     e = lap_launch_rowinfo(g->d_row_ptr, n, g->d_rowinfo, g->stream);
+    // Packed arcs where they stay in L2 (an allocation that fails leaves the
+    // plain columns).
+    if (e == cudaSuccess && n <= (1 << 21) && 8ull * (uint64_t)last <= kL2Graph) {
+        if (dalloc(&g->d_arcs, (size_t)last) != cudaSuccess) {
+            cudaGetLastError();
+            g->d_arcs = nullptr;
+        } else {
+            e = lap_launch_pack_arcs(g->d_rowinfo, g->d_col, n, last, g->d_arcs, g->stream);
+        }
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
     if (e != cudaSuccess) {
         lap_status s = cuda_fail(nullptr, e, "row records");
@@ -491,6 +546,7 @@ lap_status lap_set_workspace(lap_graph *g, void *device_ptr, uint64_t bytes)
     g->ws_bytes = bytes & ~255ull;
     g->ws_owned = false;
     g->ws_zeroed = false;
+    g->blk_clean = 0;
     g->last_kernel = 0;
     return LAP_OK;
 }
@@ -604,8 +660,11 @@ static lap_status sample_chunk(lap_graph *g, uint64_t n_samples, uint64_t seed, 
     if (g->cursor + n_samples > (1ull << 32)) return fail(g, LAP_ERR_TOO_LARGE, "sample ids are limited to 2^32");
     if (n_samples == 0) return LAP_OK;
     if ((s = resolve_pending(g)) != LAP_OK) return s;
-    const int kernel = choose_kernel(g, n_samples);
-    if ((s = ensure_workspace(g, kernel)) != LAP_OK) return s;
+    LapBlockPlan plan;
+    if (!g->ws && (s = ensure_workspace(g, LAP_KERNEL_GROUP)) != LAP_OK) return s;
+    const bool block = choose_block(g, n_samples, &plan);
+    const int kernel = block ? LAP_KERNEL_GROUP : choose_kernel(g, n_samples);
+    if (!block && (s = ensure_workspace(g, kernel)) != LAP_OK) return s;
     g->seed = seed;
     g->seed_set = true;
     g->used_kernel = kernel;
@@ -653,10 +712,13 @@ static lap_status sample_chunk(lap_graph *g, uint64_t n_samples, uint64_t seed, 
         }
         p.ovf_ids = g->d_ovf_ids;
     }
-    if ((s = launch(g, p, kernel)) != LAP_OK) return s;
+    if ((s = block ? launch_block(g, p, plan) : launch(g, p, kernel)) != LAP_OK) return s;
     if (kernel == LAP_KERNEL_COMPACT || kernel == LAP_KERNEL_GROUP) {
         g->pending = true;
         g->pending_launch = p;
+        // The block kernel's absorbed walks do not depend on a sample's Wilson
+        // run: they stand when it is withdrawn.
+        if (block) g->pending_launch.flags |= LAP_SAMPLE_WILSON_ONLY;
     }
     g->omega += n_samples;
     g->cursor += n_samples;

@@ -34,7 +34,7 @@ struct LapDevAcc {
     unsigned int status;           // LAP_DEV_* bits
     unsigned int claim;            // next sample offset to claim inside a launch
     unsigned int ovf_count;        // compact kernel: samples withdrawn in this launch
-    unsigned int pad0;
+    unsigned int walk_claim;       // block kernel: next absorbed walk to claim inside a launch
     unsigned long long pad[4];
 };
 
@@ -92,7 +92,7 @@ struct LapSampleLaunch {
 enum : uint32_t {
     LAP_SAMPLE_ONE_PER_LANE = 1u,   // lane j runs exactly sample first + j (j < count), so its
                                     // slot ends holding that sample's tree (Next of every node)
-    LAP_SAMPLE_WILSON_ONLY = 2u,    // skip the two absorbed walks (Y2 = 0, no cnt2 passes)
+    LAP_SAMPLE_WILSON_ONLY = 2u,    // skip the two absorbed walks (no cnt2 passes, Y2 and M2 not written)
 };
 cudaError_t lap_launch_sample(const LapSampleLaunch &p, cudaStream_t st);
 // sampler_compact.cu
@@ -100,6 +100,50 @@ cudaError_t lap_launch_sample_compact(const LapSampleLaunch &p, cudaStream_t st)
 // sampler_group.cu: `walkers` lanes per sample (2, 4, 8 or 16); p.slots counts groups;
 // p.stack_cap is the stack capacity of each walker
 cudaError_t lap_launch_sample_group(const LapSampleLaunch &p, int walkers, cudaStream_t st);
+
+// sampler_block.cu: a CTA per sample, the tree bits in shared memory
+struct LapBlockLaunch {
+    const unsigned long long *arcs;   // packed arcs (lap_launch_pack_arcs), or NULL
+    uint32_t bw, bo;                  // their bits of target and row offset
+    uint32_t fshift;                  // a filter bit covers 2^fshift nodes
+    uint32_t lmask;                   // lock bit of node u: u & lmask
+    uint32_t tag_base;                // sample q of the launch has tag tag_base + q + 1
+    unsigned long long *words;        // [slots * n] {tag 32 | k 32}
+    unsigned long long *path_words;   // [path_lanes * n] departures of loop-included paths
+    uint64_t path_lanes;
+    // Walkers.
+    uint32_t walk_min;                // walkers active from the start
+    float grow;                       // active walkers: grow * done^2 / n
+    uint32_t idle_min;                // idle lanes of a warp for which it looks for starts
+    uint32_t unit_batch;              // units of 32 start nodes taken at a time
+    uint32_t pair_min;                // walkers with a two-node cycle for which a warp pops them
+    uint32_t cap_a, cap_b;            // path entries of a sample's first 32 walkers, and of the others
+    uint64_t stack_entries;           // path entries of a sample
+    uint2 *stacks;                    // [slots * stack_entries] {node, k}
+    // Sweeps.
+    uint32_t sweep_nodes;             // tree size from which the sweeps run
+    uint32_t sweep_rest;              // list length that is left to the walkers
+    uint32_t *sweep;                  // [slots * 3 n] arrows, two lists
+    // Early phase (lewalk_early_kernel): samples q < early_count of the launch.
+    uint32_t early_count, early_lanes;        // samples; samples per warp
+    uint32_t early_nodes, early_budget;       // tree size and step budget at which it ends
+    uint32_t early_entries, early_log2;       // table entries of a sample
+    uint32_t early_cap;                       // path entries of a sample
+    uint32_t *early, *early_stacks, *early_pops;
+};
+struct LapBlockPlan {
+    LapBlockLaunch b = {};
+    int threads = 0;                  // Wilson threads per CTA (one more warp runs the absorbed walks)
+    uint64_t slots = 0, smem = 0;     // CTAs (samples in flight), shared memory of each
+    uint64_t words_bytes = 0;         // words and path words, zeroed when the layout grows
+    uint64_t path_offset = 0, stack_offset = 0, sweep_offset = 0, early_offset = 0;
+};
+void lap_pack_bits(int32_t n, int64_t arcs, uint32_t *bw, uint32_t *bo);
+cudaError_t lap_launch_pack_arcs(const int2 *rowinfo, const int32_t *col, int32_t n, int64_t arcs,
+                                 unsigned long long *out, cudaStream_t st);
+bool lap_block_plan(int32_t n, uint64_t count, uint64_t slots_opt, uint64_t ws_bytes, int num_sms, bool paths, bool cv,
+                    bool pack, LapBlockPlan *out);
+cudaError_t lap_launch_sample_block(const LapSampleLaunch &p, const LapBlockPlan &pl, cudaStream_t st);
 
 // ------------------------------------------------------------ batches
 // One graph of a batch (device descriptor).  Pointers index the batch's
@@ -291,6 +335,9 @@ struct lap_graph {
     uint64_t ws_bytes = 0;
     bool ws_owned = false;
     bool ws_zeroed = false;
+    unsigned long long *d_arcs = nullptr;   // packed arcs (lap_launch_pack_arcs) of graphs that keep them in L2
+    uint64_t blk_clean = 0;                 // leading workspace bytes that hold only the block kernel's tagged words
+    uint32_t tag_next = 0;                  // sample tags used since they were zeroed
 
     uint64_t step_limit = 0;                // 0: default
     uint64_t slots_opt = 0;

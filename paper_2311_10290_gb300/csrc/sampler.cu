@@ -201,6 +201,7 @@ __global__ void __launch_bounds__(256) lewalk_kernel(LapSampleLaunch p)
         } else if (phase == P_USTART) {
             if (p.flags & LAP_SAMPLE_WILSON_ONLY) {
                 acc1 += y1;
+                if (p.y1_out) p.y1_out[i - (p.ids ? p.trace_base : p.first)] = y1;
                 phase = P_CLAIM;
                 continue;
             }
