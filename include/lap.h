@@ -264,7 +264,7 @@ lap_status lap_lv_row(lap_graph *g, double *out, int out_on_device);
  * Alg. 4); b = e_s gives row s of L_v^{-1}.  b, x: n doubles, host or
  * device (on_device); iterations and residual (may be NULL) receive the
  * iterations run and the final relative residual.  Synchronises; allocates
- * and frees 4 n + 2056 doubles of device scratch.  Errors: LAP_ERR_NO_ROOT,
+ * and frees about 4 n doubles of device scratch.  Errors: LAP_ERR_NO_ROOT,
  * LAP_ERR_INVALID_ARG, LAP_ERR_OOM, LAP_ERR_CUDA.
  */
 lap_status lap_lv_solve(lap_graph *g, const double *b, double *x, int on_device, double rtol, int32_t maxiter,

@@ -12,6 +12,7 @@
 //   * the coefficients beta1, beta2 from pilot batches (least squares).
 #include "lap_internal.h"
 #include "philox.cuh"
+#include "rows.cuh"
 
 namespace {
 
@@ -27,36 +28,42 @@ int grid_for(int64_t work)
 #define NODE_LOOP(u, n) for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < (n); u += (int64_t)gridDim.x * blockDim.x)
 
 // s1[u] = sum of neighbour degrees, ones[u] = neighbours of degree 1.
-__global__ void feat_pass1(const int2 *__restrict__ rowinfo, const int32_t *__restrict__ col, int32_t n,
-                           double *__restrict__ s1, double *__restrict__ ones)
-{
-    NODE_LOOP(u, n)
+struct DegreeSums {
+    using T = lap_rows::Pair;
+    const int2 *rowinfo;
+    double *s1, *ones;
+    __device__ bool skip() const { return false; }
+    __device__ bool begin(int32_t) const { return true; }
+    __device__ T zero() const { return {0.0, 0.0}; }
+    __device__ T edge(int32_t w) const
     {
-        const int2 r = rowinfo[u];
-        double a = 0.0, b = 0.0;
-        for (int32_t e = 0; e < r.y; ++e) {
-            const int32_t d = rowinfo[col[r.x + e]].y;
-            a += (double)d;
-            b += d == 1 ? 1.0 : 0.0;
-        }
-        s1[u] = a;
-        ones[u] = b;
+        const int32_t d = rowinfo[w].y;
+        return {(double)d, d == 1 ? 1.0 : 0.0};
     }
-}
+    __device__ void end(int32_t u, int2, T t) const
+    {
+        s1[u] = t.a;
+        ones[u] = t.b;
+    }
+};
 
-// out[u] = sum over neighbours x of in[x] (optionally divided by d_u, with
-// out[v] = 1: one step of the "hit v within k steps" iteration).
-__global__ void neighbour_sum_kernel(const int2 *__restrict__ rowinfo, const int32_t *__restrict__ col, int32_t n,
-                                     const double *__restrict__ in, double *__restrict__ out, int32_t absorb_root)
+// out[u] = sum over neighbours x of in[x] (absorb >= 0: divided by d_u, with
+// out[absorb] = 1, one step of the "hit v within k steps" iteration).
+struct NeighbourSum {
+    using T = double;
+    const double *in;
+    double *out;
+    int32_t absorb;
+    __device__ bool skip() const { return false; }
+    __device__ bool begin(int32_t) const { return true; }
+    __device__ T zero() const { return 0.0; }
+    __device__ T edge(int32_t w) const { return in[w]; }
+    __device__ void end(int32_t u, int2 r, T t) const { out[u] = absorb < 0 ? t : u == absorb ? 1.0 : t / (double)r.y; }
+};
+
+__global__ void indicator_kernel(int32_t n, int32_t root, double *__restrict__ a)
 {
-    NODE_LOOP(u, n)
-    {
-        const int2 r = rowinfo[u];
-        double a = 0.0;
-        for (int32_t e = 0; e < r.y; ++e) a += in[col[r.x + e]];
-        if (absorb_root >= 0) a = (u == absorb_root) ? 1.0 : a / (double)r.y;
-        out[u] = a;
-    }
+    NODE_LOOP(u, n) a[u] = u == root ? 1.0 : 0.0;
 }
 
 __global__ void feat_assemble(const int2 *__restrict__ rowinfo, const int32_t *__restrict__ hops, int32_t n,
@@ -83,17 +90,16 @@ __global__ void quantize_kernel(const double *__restrict__ phi, int32_t n, long 
     NODE_LOOP(u, n) h[u] = __double2ll_rn(ldexp(phi[u], LAP_CV_FIXED_POINT_BITS));
 }
 
-__global__ void int_neighbour_sum_kernel(const int2 *__restrict__ rowinfo, const int32_t *__restrict__ col, int32_t n,
-                                         const long long *__restrict__ h, long long *__restrict__ S)
-{
-    NODE_LOOP(u, n)
-    {
-        const int2 r = rowinfo[u];
-        long long a = 0;
-        for (int32_t e = 0; e < r.y; ++e) a += h[col[r.x + e]];
-        S[u] = a;
-    }
-}
+struct IntNeighbourSum {
+    using T = long long;
+    const long long *h;
+    long long *S;
+    __device__ bool skip() const { return false; }
+    __device__ bool begin(int32_t) const { return true; }
+    __device__ T zero() const { return 0; }
+    __device__ T edge(int32_t w) const { return h[w]; }
+    __device__ void end(int32_t u, int2, T t) const { S[u] = t; }
+};
 
 // One thread per (node, repetition): a walk from u absorbed at v; step t uses
 // Philox counter (t, u, rep, 3).
@@ -404,36 +410,31 @@ cudaError_t lap_launch_beta2_reduce(const unsigned long long *y1, const unsigned
     return cudaGetLastError();
 }
 
-cudaError_t lap_launch_features(const int2 *rowinfo, const int32_t *col, const int32_t *hops, int32_t n, int32_t root,
-                                double *scratch /* 5 n */, float *feat, cudaStream_t st)
+cudaError_t lap_launch_features(const int2 *rowinfo, const int32_t *col, const int32_t *hops, int32_t n, LapHubs hubs,
+                                int32_t root, double *scratch /* 5 n */, float *feat, cudaStream_t st)
 {
     double *s1 = scratch, *ones = scratch + n, *s2 = scratch + 2 * (int64_t)n, *a = scratch + 3 * (int64_t)n,
            *b = scratch + 4 * (int64_t)n;
     const int grid = grid_for(n);
-    feat_pass1<<<grid, kBlock, 0, st>>>(rowinfo, col, n, s1, ones);
-    neighbour_sum_kernel<<<grid, kBlock, 0, st>>>(rowinfo, col, n, s1, s2, -1);
-    cudaError_t e = cudaMemsetAsync(a, 0, sizeof(double) * (size_t)n, st);
+    cudaError_t e = lap_rows::launch_rows(DegreeSums{rowinfo, s1, ones}, rowinfo, col, n, hubs, st);
+    if (e == cudaSuccess) e = lap_rows::launch_rows(NeighbourSum{s1, s2, -1}, rowinfo, col, n, hubs, st);
     if (e != cudaSuccess) return e;
-    const double one = 1.0;
-    e = cudaMemcpyAsync(a + root, &one, sizeof(double), cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return e;
+    indicator_kernel<<<grid, kBlock, 0, st>>>(n, root, a);
     for (int it = 0; it < LAP_CV_ABSORB_ITERS; ++it) {
-        neighbour_sum_kernel<<<grid, kBlock, 0, st>>>(rowinfo, col, n, a, b, root);
+        if ((e = lap_rows::launch_rows(NeighbourSum{a, b, root}, rowinfo, col, n, hubs, st)) != cudaSuccess) return e;
         double *t = a; a = b; b = t;
     }
     feat_assemble<<<grid, kBlock, 0, st>>>(rowinfo, hops, n, s1, s2, ones, a, feat);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return cudaStreamSynchronize(st);   // the host constant above must outlive the copy
+    return cudaStreamSynchronize(st);
 }
 
-cudaError_t lap_launch_potential(const int2 *rowinfo, const int32_t *col, int32_t n, const double *phi, long long *h,
-                                 long long *S, cudaStream_t st)
+cudaError_t lap_launch_potential(const int2 *rowinfo, const int32_t *col, int32_t n, LapHubs hubs, const double *phi,
+                                 long long *h, long long *S, cudaStream_t st)
 {
-    const int grid = grid_for(n);
-    quantize_kernel<<<grid, kBlock, 0, st>>>(phi, n, h);
-    int_neighbour_sum_kernel<<<grid, kBlock, 0, st>>>(rowinfo, col, n, h, S);
-    return cudaGetLastError();
+    quantize_kernel<<<grid_for(n), kBlock, 0, st>>>(phi, n, h);
+    return lap_rows::launch_rows(IntNeighbourSum{h, S}, rowinfo, col, n, hubs, st);
 }
 
 cudaError_t lap_launch_hitting_walks(const LapDevGraph &g, int32_t root, uint64_t seed, uint32_t reps, uint64_t limit,

@@ -5,6 +5,7 @@
 // checks connectivity (Section 2 assumes G connected; Wilson's algorithm does
 // not terminate otherwise) and records hop distances.
 #include "lap_internal.h"
+#include "rows.cuh"
 
 namespace {
 
@@ -86,6 +87,46 @@ __global__ void argmax_degree_kernel(const int2 *__restrict__ rowinfo, int32_t n
     if ((threadIdx.x & 31) == 0) atomicMax(best, m);
 }
 
+__global__ void find_hubs_kernel(const int2 *__restrict__ rowinfo, int32_t n, int32_t *__restrict__ ids, unsigned int *count)
+{
+    for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n; u += (int64_t)gridDim.x * blockDim.x)
+        if (rowinfo[u].y > LAP_HUB_DEGREE) ids[atomicAdd(count, 1u)] = (int32_t)u;
+}
+
+__global__ void bfs_start_kernel(int32_t *hops, int32_t n, int32_t root, unsigned int *flags)
+{
+    for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n; u += (int64_t)gridDim.x * blockDim.x)
+        hops[u] = (u == root) ? 0 : -1;
+    if (blockIdx.x == 0 && threadIdx.x == 0) flags[0] = 1u;
+}
+
+// One level: flag[0] says whether any node has it, flag[1] is set when a node
+// is found.  A neighbour that has its hops already (most) is only read.
+struct BfsLevel {
+    using T = unsigned int;
+    int32_t *hops;
+    unsigned int *flag;
+    int32_t level;
+    __device__ bool skip() const { return *flag == 0u; }
+    __device__ bool begin(int32_t u) const { return hops[u] == level; }
+    __device__ T zero() const { return 0u; }
+    __device__ T edge(int32_t w) const { return hops[w] == -1 && atomicCAS(&hops[w], -1, level + 1) == -1 ? 1u : 0u; }
+    __device__ void end(int32_t, int2, T found) const
+    {
+        if (found) flag[1] = 1u;
+    }
+};
+
+__global__ void count_reached_kernel(const int32_t *__restrict__ hops, int32_t n, unsigned int *count)
+{
+    unsigned int got = 0;
+    for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n; u += (int64_t)gridDim.x * blockDim.x)
+        got += hops[u] >= 0;
+    got = __reduce_add_sync(0xFFFFFFFFu, got);
+    if ((threadIdx.x & 31) == 0 && got) atomicAdd(count, got);
+}
+
+// Batches of graphs: one thread per row, all graphs' levels queued together.
 __global__ void bfs_init_kernel(int32_t *hops, int32_t n, int32_t root)
 {
     for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n; u += (int64_t)gridDim.x * blockDim.x)
@@ -133,6 +174,36 @@ cudaError_t lap_launch_argmax_degree(const int2 *rowinfo, int32_t n, unsigned lo
 {
     argmax_degree_kernel<<<grid_for(n, kBlock), kBlock, 0, st>>>(rowinfo, n, best);
     return cudaGetLastError();
+}
+
+cudaError_t lap_launch_find_hubs(const int2 *rowinfo, int32_t n, int32_t *ids, unsigned int *count, cudaStream_t st)
+{
+    find_hubs_kernel<<<grid_for(n, kBlock), kBlock, 0, st>>>(rowinfo, n, ids, count);
+    return cudaGetLastError();
+}
+
+cudaError_t lap_run_bfs(const int2 *rowinfo, const int32_t *col, int32_t n, LapHubs hubs, int32_t root, int32_t *hops,
+                        unsigned int *flags, int64_t *reached, cudaStream_t st)
+{
+    // Levels are queued kLevels at a time and the host looks once per batch; a
+    // level that no node has returns at once.
+    constexpr int kLevels = 8;
+    cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(unsigned int) * (kLevels + 2), st);
+    if (e != cudaSuccess) return e;
+    bfs_start_kernel<<<grid_for(n, kBlock), kBlock, 0, st>>>(hops, n, root, flags);
+    for (int32_t base = 0;; base += kLevels) {
+        for (int32_t l = 0; l < kLevels; ++l) {
+            e = lap_rows::launch_rows(BfsLevel{hops, flags + l, base + l}, rowinfo, col, n, hubs, st);
+            if (e != cudaSuccess) return e;
+        }
+        count_reached_kernel<<<grid_for(n, kBlock), kBlock, 0, st>>>(hops, n, flags + kLevels + 1);
+        unsigned int h[2] = {0, 0};
+        if ((e = cudaMemcpyAsync(h, flags + kLevels, sizeof(h), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
+        if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
+        *reached = h[1];
+        if (h[0] == 0) return cudaGetLastError();
+        if ((e = cudaMemsetAsync(flags + 1, 0, sizeof(unsigned int) * (kLevels + 1), st)) != cudaSuccess) return e;   // flags[0] stays 1
+    }
 }
 
 cudaError_t lap_launch_bfs_init(int32_t *hops, int32_t n, int32_t root, cudaStream_t st)

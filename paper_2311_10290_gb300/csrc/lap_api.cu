@@ -1,5 +1,6 @@
 // Host side of the C ABI declared in include/lap.h: argument checks, device
 // memory of a handle, stream handling, launch sizing and error reporting.
+#include <algorithm>
 #include <atomic>
 #include <cstdio>
 #include <cstring>
@@ -45,6 +46,7 @@ void free_all(lap_graph *g)
     cudaFree(g->d_col);
     cudaFree(g->d_rowinfo);
     cudaFree(g->d_arcs);
+    cudaFree(g->d_hubs);
     cudaFree(g->d_hops);
     cudaFree(g->d_rep1);
     cudaFree(g->d_cnt2);
@@ -420,6 +422,28 @@ lap_status lap_graph_create(int32_t n, const int32_t *row_ptr, const int32_t *co
         return bad;
     }
     e = lap_launch_rowinfo(g->d_row_ptr, n, g->d_rowinfo, g->stream);
+    // Hubs, in id order (the row kernels' sums keep one order).
+    unsigned int hub_count = 0;
+    if (e == cudaSuccess && dalloc(&g->d_hubs, (size_t)(last / LAP_HUB_DEGREE) + 1) != cudaSuccess) {
+        cudaGetLastError();
+        free_all(g);
+        delete g;
+        return fail(nullptr, LAP_ERR_OOM, "device allocation failed");
+    }
+    if (e == cudaSuccess) e = cudaMemsetAsync(&g->d_acc->claim, 0, sizeof(unsigned int), g->stream);
+    if (e == cudaSuccess) e = lap_launch_find_hubs(g->d_rowinfo, n, g->d_hubs, &g->d_acc->claim, g->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&hub_count, &g->d_acc->claim, sizeof(hub_count), cudaMemcpyDeviceToHost, g->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
+    if (e == cudaSuccess && hub_count) {
+        std::vector<int32_t> ids(hub_count);
+        const size_t bytes = sizeof(int32_t) * hub_count;
+        e = cudaMemcpyAsync(ids.data(), g->d_hubs, bytes, cudaMemcpyDeviceToHost, g->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
+        std::sort(ids.begin(), ids.end());
+        if (e == cudaSuccess) e = cudaMemcpyAsync(g->d_hubs, ids.data(), bytes, cudaMemcpyHostToDevice, g->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
+    }
+    g->hubs = LapHubs{g->d_hubs, (int32_t)hub_count};
     // Packed arcs where they stay in L2 (an allocation that fails leaves the
     // plain columns).
     if (e == cudaSuccess && n <= (1 << 21) && 8ull * (uint64_t)last <= kL2Graph) {
@@ -567,18 +591,9 @@ lap_status lap_set_root(lap_graph *g, int32_t v, int32_t *root_out)
         v = (int32_t)(0xFFFFFFFFu - (uint32_t)(h & 0xFFFFFFFFull));
     }
     // Breadth-first search from v: connectivity check and hop distances.
-    unsigned int *found = reinterpret_cast<unsigned int *>(g->d_red);
-    LAP_CUDA(g, lap_launch_bfs_init(g->d_hops, g->n, v, g->stream));
-    int64_t reached = 1;
-    for (int32_t level = 0;; ++level) {
-        LAP_CUDA(g, cudaMemsetAsync(found, 0, sizeof(unsigned int), g->stream));
-        LAP_CUDA(g, lap_launch_bfs_level(g->d_rowinfo, g->d_col, g->d_hops, g->n, level, found, g->stream));
-        unsigned int h = 0;
-        LAP_CUDA(g, cudaMemcpyAsync(&h, found, sizeof(h), cudaMemcpyDeviceToHost, g->stream));
-        LAP_CUDA(g, cudaStreamSynchronize(g->stream));
-        if (h == 0) break;
-        reached += h;
-    }
+    int64_t reached = 0;
+    LAP_CUDA(g, lap_run_bfs(g->d_rowinfo, g->d_col, g->n, g->hubs, v, g->d_hops, reinterpret_cast<unsigned int *>(g->d_red),
+                            &reached, g->stream));
     if (reached != g->n) {
         char buf[160];
         snprintf(buf, sizeof(buf), "root %d reaches %lld of %d nodes: graph is not connected", v, (long long)reached, g->n);
@@ -838,7 +853,7 @@ lap_status lap_lv_solve(lap_graph *g, const double *b, double *x, int on_device,
         cudaFree(db);
         cudaFree(dx);
     };
-    bool ok = dalloc(&scratch, 4 * n + 2 * 1024 + 8) == cudaSuccess;
+    bool ok = dalloc(&scratch, (size_t)lap_lv_solve_scratch(g->n, g->hubs)) == cudaSuccess;
     if (ok && !on_device) ok = dalloc(&db, n) == cudaSuccess && dalloc(&dx, n) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -850,7 +865,7 @@ lap_status lap_lv_solve(lap_graph *g, const double *b, double *x, int on_device,
     int32_t it = 0;
     double res = 0.0;
     if (e == cudaSuccess)
-        e = lap_run_lv_solve(g->d_rowinfo, g->d_col, g->n, g->root, on_device ? b : db, on_device ? x : dx, scratch,
+        e = lap_run_lv_solve(g->d_rowinfo, g->d_col, g->n, g->hubs, g->root, on_device ? b : db, on_device ? x : dx, scratch,
                              rtol, maxiter, &it, &res, g->stream);
     if (e == cudaSuccess && !on_device) e = cudaMemcpyAsync(x, dx, sizeof(double) * n, cudaMemcpyDeviceToHost, g->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
@@ -1131,7 +1146,7 @@ lap_status lap_features(lap_graph *g, float *feat_dev)
         cudaGetLastError();
         return fail(g, LAP_ERR_OOM, "feature scratch allocation failed");
     }
-    LAP_CUDA(g, lap_launch_features(g->d_rowinfo, g->d_col, g->d_hops, g->n, g->root, g->d_feat_scratch, feat_dev,
+    LAP_CUDA(g, lap_launch_features(g->d_rowinfo, g->d_col, g->d_hops, g->n, g->hubs, g->root, g->d_feat_scratch, feat_dev,
                                     g->stream));
     return LAP_OK;
 }
@@ -1301,8 +1316,8 @@ lap_status lap_cv_set_potentials(lap_graph *g, const double *phi1_dev, const dou
     }
     g->cv1 = phi1_dev != nullptr;
     g->cv2 = phi2_dev != nullptr;
-    if (phi1_dev) LAP_CUDA(g, lap_launch_potential(g->d_rowinfo, g->d_col, g->n, phi1_dev, g->d_cv_h1, g->d_cv_S1, g->stream));
-    if (phi2_dev) LAP_CUDA(g, lap_launch_potential(g->d_rowinfo, g->d_col, g->n, phi2_dev, g->d_cv_h2, g->d_cv_S2, g->stream));
+    if (phi1_dev) LAP_CUDA(g, lap_launch_potential(g->d_rowinfo, g->d_col, g->n, g->hubs, phi1_dev, g->d_cv_h1, g->d_cv_S1, g->stream));
+    if (phi2_dev) LAP_CUDA(g, lap_launch_potential(g->d_rowinfo, g->d_col, g->n, g->hubs, phi2_dev, g->d_cv_h2, g->d_cv_S2, g->stream));
     g->results_valid = false;
     return LAP_OK;
 }

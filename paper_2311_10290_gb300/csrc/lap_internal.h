@@ -38,6 +38,14 @@ struct LapDevAcc {
     unsigned long long pad[4];
 };
 
+// Nodes of more than LAP_HUB_DEGREE neighbours, ascending: the row kernels
+// (rows.cuh) give each a CTA.
+constexpr int32_t LAP_HUB_DEGREE = 256;
+struct LapHubs {
+    const int32_t *ids;    // device
+    int32_t count;
+};
+
 // ---------------------------------------------------------------- kernels
 // ingest.cu
 cudaError_t lap_launch_validate(const int32_t *row_ptr, const int32_t *col, int32_t n, int64_t arcs,
@@ -47,6 +55,12 @@ cudaError_t lap_launch_argmax_degree(const int2 *rowinfo, int32_t n, unsigned lo
 cudaError_t lap_launch_bfs_init(int32_t *hops, int32_t n, int32_t root, cudaStream_t st);
 cudaError_t lap_launch_bfs_level(const int2 *rowinfo, const int32_t *col, int32_t *hops, int32_t n,
                                  int32_t level, unsigned int *found, cudaStream_t st);
+// ids[0..*count) in any order (at most arcs / LAP_HUB_DEGREE of them)
+cudaError_t lap_launch_find_hubs(const int2 *rowinfo, int32_t n, int32_t *ids, unsigned int *count, cudaStream_t st);
+// Breadth-first search from `root`: hops (-1: not reached) and the number of
+// nodes reached; flags: 16 unsigned ints of device scratch.
+cudaError_t lap_run_bfs(const int2 *rowinfo, const int32_t *col, int32_t n, LapHubs hubs, int32_t root, int32_t *hops,
+                        unsigned int *flags, int64_t *reached, cudaStream_t st);
 
 // sampler.cu
 struct LapSampleLaunch {
@@ -201,10 +215,11 @@ struct LapBatchLaunch {
 cudaError_t lap_launch_batch(const LapBatchLaunch &p, bool probe, cudaStream_t st);
 int lap_batch_block(const LapBatchLaunch &p);
 uint64_t lap_batch_resident_lanes(int block, int num_sms);
-// solve.cu: conjugate gradients for L_v x = b; scratch: 4 n + 2 * 1024 + 8 doubles
-cudaError_t lap_run_lv_solve(const int2 *rowinfo, const int32_t *col, int32_t n, int32_t v, const double *b, double *x,
-                             double *scratch, double rtol, int32_t maxiter, int32_t *iterations, double *residual,
-                             cudaStream_t st);
+// solve.cu: conjugate gradients for L_v x = b
+uint64_t lap_lv_solve_scratch(int32_t n, LapHubs hubs);       // doubles of scratch
+cudaError_t lap_run_lv_solve(const int2 *rowinfo, const int32_t *col, int32_t n, LapHubs hubs, int32_t v,
+                             const double *b, double *x, double *scratch, double rtol, int32_t maxiter,
+                             int32_t *iterations, double *residual, cudaStream_t st);
 
 // finalize.cu: finalize of every graph of a batch, bit-identical per graph to
 // lap_launch_finalize; red holds graphs * (1024 + 2) doubles.
@@ -259,9 +274,9 @@ inline uint32_t lap_table_log2(int64_t n)
 // Control variate (cv.cu, mlp.cu).
 constexpr int LAP_CV_FIXED_POINT_BITS = 16;   // h = round(2^16 phi)
 constexpr int LAP_CV_ABSORB_ITERS = 8;        // feature f7: P(hit v within 8 steps)
-cudaError_t lap_launch_features(const int2 *rowinfo, const int32_t *col, const int32_t *hops, int32_t n, int32_t root,
+cudaError_t lap_launch_features(const int2 *rowinfo, const int32_t *col, const int32_t *hops, int32_t n, LapHubs hubs, int32_t root,
                                 double *scratch, float *feat, cudaStream_t st);
-cudaError_t lap_launch_potential(const int2 *rowinfo, const int32_t *col, int32_t n, const double *phi, long long *h,
+cudaError_t lap_launch_potential(const int2 *rowinfo, const int32_t *col, int32_t n, LapHubs hubs, const double *phi, long long *h,
                                  long long *S, cudaStream_t st);
 cudaError_t lap_launch_hitting_walks(const LapDevGraph &g, int32_t root, uint64_t seed, uint32_t reps, uint64_t limit,
                                      unsigned long long *sums, unsigned int *status, int num_sms, cudaStream_t st);
@@ -313,6 +328,8 @@ struct lap_graph {
     int32_t *d_col = nullptr;
     int2 *d_rowinfo = nullptr;
     int32_t *d_hops = nullptr;
+    int32_t *d_hubs = nullptr;
+    LapHubs hubs = {nullptr, 0};
     unsigned long long *d_rep1 = nullptr;   // repeat visits per node (visits - 1, summed)
     unsigned long long *d_cnt2 = nullptr;   // uniform-start walk passes per node
     LapDevAcc *d_acc = nullptr;
