@@ -244,46 +244,35 @@ lap_status launch(lap_graph *g, LapSampleLaunch &p, int kernel)
     return LAP_OK;
 }
 
-constexpr int32_t kBlockMinNodes = 2048;
-
-// The block kernel (sampler_block.cu) takes automatic calls and kernel 3 with
-// the automatic number of walkers, where it applies: `pl` is the launch then.
-bool choose_block(const lap_graph *g, uint64_t n_samples, LapBlockPlan *pl)
+// Automatic calls, and kernel 3 with the automatic number of walkers, take the
+// kernels that run a sample's Wilson run and its absorbed walks in different
+// warps (sampler_cta.cu), where they apply.
+bool choose_cta(const lap_graph *g, uint64_t n_samples, LapCtaPlan *pl)
 {
-    if (g->walkers || g->compact_disabled || !g->ws || (g->kernel_opt == 0 && g->n < kBlockMinNodes)) return false;
+    if (g->walkers || g->compact_disabled || !g->ws) return false;
     if (g->kernel_opt != 0 && g->kernel_opt != LAP_KERNEL_GROUP) return false;
-    return lap_block_plan(g->n, n_samples, g->slots_opt, g->ws_bytes, g->num_sms, g->paths_opt != 0, g->cv1 || g->cv2,
-                          g->d_arcs != nullptr, pl);
+    return lap_cta_plan(g->n, g->arcs, n_samples, g->slots_opt, g->ws_bytes, g->num_sms, g->paths_opt != 0, g->cv1 || g->cv2,
+                        g->d_arcs != nullptr, pl);
 }
 
-lap_status launch_block(lap_graph *g, LapSampleLaunch &p, LapBlockPlan &pl)
+lap_status launch_cta(lap_graph *g, LapSampleLaunch &p, LapCtaPlan &pl)
 {
     // The tagged words are zeroed when the workspace last held something else
     // there, and when the tags (31 bits) run out.
-    if (pl.words_bytes > g->blk_clean || (uint64_t)g->tag_next + p.count + 1ull >= (1ull << 31)) {
-        LAP_CUDA(g, cudaMemsetAsync(g->ws, 0, pl.words_bytes, g->stream));
+    const uint64_t words = pl.words_bytes();
+    if (words > g->blk_clean || (uint64_t)g->tag_next + p.count + 1ull >= (1ull << 31)) {
+        LAP_CUDA(g, cudaMemsetAsync(g->ws, 0, words, g->stream));
         g->tag_next = 0;
     }
-    g->blk_clean = pl.words_bytes;
+    g->blk_clean = words;
     g->last_kernel = LAP_KERNEL_GROUP;
     g->ws_zeroed = false;
-    uint8_t *ws = reinterpret_cast<uint8_t *>(g->ws);
-    p.slots = pl.slots;
-    pl.b.arcs = g->d_arcs;
-    if (g->d_arcs) lap_pack_bits(g->n, g->arcs, &pl.b.bw, &pl.b.bo);
-    pl.b.tag_base = g->tag_next;
-    pl.b.words = reinterpret_cast<unsigned long long *>(ws);
-    pl.b.path_words = reinterpret_cast<unsigned long long *>(ws + pl.path_offset);
-    pl.b.stacks = reinterpret_cast<uint2 *>(ws + pl.stack_offset);
-    pl.b.sweep = reinterpret_cast<uint32_t *>(ws + pl.sweep_offset);
-    pl.b.early = reinterpret_cast<uint32_t *>(ws + pl.early_offset);
-    pl.b.early_stacks = pl.b.early + (uint64_t)pl.b.early_entries * pl.b.early_count;
-    pl.b.early_pops = pl.b.early_stacks + (uint64_t)pl.b.early_cap * pl.b.early_count;
+    const uint32_t tag = g->tag_next;
     g->tag_next += p.count;
     LAP_CUDA(g, cudaMemsetAsync(&g->d_acc->claim, 0, sizeof(unsigned int), g->stream));
     LAP_CUDA(g, cudaMemsetAsync(&g->d_acc->walk_claim, 0, sizeof(unsigned int), g->stream));
-    const cudaError_t e = lap_launch_sample_block(p, pl, g->stream);
-    if (e != cudaSuccess) return cuda_fail(g, e, "sampler launch (block kernel)");
+    const cudaError_t e = lap_launch_cta(p, pl, g->ws, g->d_arcs, tag, g->stream);
+    if (e != cudaSuccess) return cuda_fail(g, e, "sampler launch (kernel 3)");
     return LAP_OK;
 }
 
@@ -675,11 +664,11 @@ static lap_status sample_chunk(lap_graph *g, uint64_t n_samples, uint64_t seed, 
     if (g->cursor + n_samples > (1ull << 32)) return fail(g, LAP_ERR_TOO_LARGE, "sample ids are limited to 2^32");
     if (n_samples == 0) return LAP_OK;
     if ((s = resolve_pending(g)) != LAP_OK) return s;
-    LapBlockPlan plan;
+    LapCtaPlan plan;
     if (!g->ws && (s = ensure_workspace(g, LAP_KERNEL_GROUP)) != LAP_OK) return s;
-    const bool block = choose_block(g, n_samples, &plan);
-    const int kernel = block ? LAP_KERNEL_GROUP : choose_kernel(g, n_samples);
-    if (!block && (s = ensure_workspace(g, kernel)) != LAP_OK) return s;
+    const bool cta = choose_cta(g, n_samples, &plan);
+    const int kernel = cta ? LAP_KERNEL_GROUP : choose_kernel(g, n_samples);
+    if (!cta && (s = ensure_workspace(g, kernel)) != LAP_OK) return s;
     g->seed = seed;
     g->seed_set = true;
     g->used_kernel = kernel;
@@ -727,13 +716,13 @@ static lap_status sample_chunk(lap_graph *g, uint64_t n_samples, uint64_t seed, 
         }
         p.ovf_ids = g->d_ovf_ids;
     }
-    if ((s = block ? launch_block(g, p, plan) : launch(g, p, kernel)) != LAP_OK) return s;
+    if ((s = cta ? launch_cta(g, p, plan) : launch(g, p, kernel)) != LAP_OK) return s;
     if (kernel == LAP_KERNEL_COMPACT || kernel == LAP_KERNEL_GROUP) {
         g->pending = true;
         g->pending_launch = p;
-        // The block kernel's absorbed walks do not depend on a sample's Wilson
-        // run: they stand when it is withdrawn.
-        if (block) g->pending_launch.flags |= LAP_SAMPLE_WILSON_ONLY;
+        // These kernels' absorbed walks do not depend on a sample's Wilson run:
+        // they stand when it is withdrawn.
+        if (cta) g->pending_launch.flags |= LAP_SAMPLE_WILSON_ONLY;
     }
     g->omega += n_samples;
     g->cursor += n_samples;

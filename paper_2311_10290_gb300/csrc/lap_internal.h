@@ -137,7 +137,7 @@ struct LapBlockLaunch {
     // Sweeps.
     uint32_t sweep_nodes;             // tree size from which the sweeps run
     uint32_t sweep_rest;              // list length that is left to the walkers
-    uint32_t *sweep;                  // [slots * 3 n] arrows, two lists
+    uint32_t *sweep;                  // [slots * 3 n] arrows, two lists; small graphs: [slots * n] draws beyond 254
     // Early phase (lewalk_early_kernel): samples q < early_count of the launch.
     uint32_t early_count, early_lanes;        // samples; samples per warp
     uint32_t early_nodes, early_budget;       // tree size and step budget at which it ends
@@ -158,6 +158,31 @@ cudaError_t lap_launch_pack_arcs(const int2 *rowinfo, const int32_t *col, int32_
 bool lap_block_plan(int32_t n, uint64_t count, uint64_t slots_opt, uint64_t ws_bytes, int num_sms, bool paths, bool cv,
                     bool pack, LapBlockPlan *out);
 cudaError_t lap_launch_sample_block(const LapSampleLaunch &p, const LapBlockPlan &pl, cudaStream_t st);
+
+// sampler_small.cu: a lane per sample, state and graph in shared memory
+struct LapSmallPlan {
+    LapBlockLaunch b = {};            // arcs, path words, stacks, tags
+    int warps = 0;                    // per CTA (one more runs the absorbed walks)
+    uint32_t lanes = 0;               // lanes of a warp that take samples
+    bool local = false;               // the graph is copied to shared memory
+    uint64_t slots = 0, blocks = 0, smem = 0, words_bytes = 0, stack_offset = 0, many_offset = 0;
+};
+bool lap_small_plan(int32_t n, int64_t arcs, uint64_t count, uint64_t slots_opt, uint64_t ws_bytes, int num_sms, bool paths,
+                    LapSmallPlan *out);
+cudaError_t lap_launch_sample_small(const LapSampleLaunch &p, const LapSmallPlan &pl, cudaStream_t st);
+
+// sampler_cta.cu: the launch of a call by one of these two kernels
+struct LapCtaPlan {
+    bool small = false;
+    LapBlockPlan block;
+    LapSmallPlan lane;
+    uint64_t words_bytes() const { return small ? lane.words_bytes : block.words_bytes; }
+};
+bool lap_cta_plan(int32_t n, int64_t arcs, uint64_t count, uint64_t slots_opt, uint64_t ws_bytes, int num_sms, bool paths,
+                  bool cv, bool pack, LapCtaPlan *out);
+// ws: its first words_bytes() hold zeros, or words of this layout under other tags
+cudaError_t lap_launch_cta(LapSampleLaunch &p, LapCtaPlan &pl, void *ws, const unsigned long long *arcs, uint32_t tag_base,
+                           cudaStream_t st);
 
 // ------------------------------------------------------------ batches
 // One graph of a batch (device descriptor).  Pointers index the batch's
