@@ -1002,6 +1002,72 @@ static lap_status spantree_prepare(lap_graph *g)
     return LAP_OK;
 }
 
+static lap_status spantree_failed(lap_graph *g, unsigned int status)
+{
+    if (status & LAP_DEV_STEP_LIMIT) {
+        g->sticky = LAP_ERR_STEP_LIMIT;
+        return fail(g, LAP_ERR_STEP_LIMIT, "a Wilson run exceeded the per-sample step budget (LAP_OPT_STEP_LIMIT)");
+    }
+    g->sticky = LAP_ERR_CUDA;
+    return fail(g, LAP_ERR_CUDA, "internal error in the SpanTree kernels (status " + std::to_string(status) + ")");
+}
+
+// Samples up to n_samples trees with the block kernel, half of the workspace
+// for its state and the rest for the trees; *c: how many (0: it does not fit, or
+// a sample was withdrawn).
+static lap_status spantree_block(lap_graph *g, LapSampleLaunch &p, uint64_t n_samples, uint64_t *c, LapSpanTreeLaunch *t)
+{
+    const uint64_t per_tree = 4ull * (uint64_t)g->n, half = (g->ws_bytes / 2ull) & ~255ull;
+    *c = 0;
+    if (g->compact_disabled || (g->kernel_opt != 0 && g->kernel_opt != LAP_KERNEL_GROUP)) return LAP_OK;
+    uint64_t m = (g->ws_bytes - half) / per_tree;
+    if (m > n_samples) m = n_samples;
+    if (m > (1ull << 24)) m = 1ull << 24;
+    LapCtaPlan pl;
+    if (m == 0 || !lap_block_plan(g->n, m, g->slots_opt, half, g->num_sms, false, false, g->d_arcs != nullptr, &pl.block))
+        return LAP_OK;
+    g->last_kernel = LAP_KERNEL_GROUP;
+    g->ws_zeroed = false;
+    g->blk_clean = 0;
+    LAP_CUDA(g, cudaMemsetAsync(g->ws, 0, pl.words_bytes(), g->stream));
+    LAP_CUDA(g, cudaMemsetAsync(&g->d_st_acc->claim, 0, sizeof(unsigned int), g->stream));
+    LAP_CUDA(g, cudaMemsetAsync(&g->d_st_acc->ovf_count, 0, sizeof(unsigned int), g->stream));
+    p.count = (uint32_t)m;
+    p.flags = LAP_SAMPLE_WILSON_ONLY;
+    p.tree_out = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(g->ws) + half);
+    LAP_CUDA(g, lap_launch_cta(p, pl, g->ws, g->d_arcs, 0u, g->stream));
+    LapDevAcc h;
+    LAP_CUDA(g, cudaMemcpyAsync(&h, g->d_st_acc, sizeof(h), cudaMemcpyDeviceToHost, g->stream));
+    LAP_CUDA(g, cudaStreamSynchronize(g->stream));
+    if (h.ovf_count) return LAP_OK;                  // these trees again, with the other kernel
+    // (After a status bit the trees are undefined; the caller reports it.)
+    *c = m;
+    t->trees = p.tree_out;
+    t->tree_stride = 1;
+    return h.status ? spantree_failed(g, h.status) : LAP_OK;
+}
+
+// The same with the 8-byte kernel, a lane per tree.
+static lap_status spantree_wide(lap_graph *g, LapSampleLaunch &p, uint64_t n_samples, uint64_t *c, LapSpanTreeLaunch *t)
+{
+    lap_status s = ensure_workspace(g, LAP_KERNEL_WIDE);
+    if (s != LAP_OK) return s;
+    uint64_t cap = g->ws_bytes / (8ull * (uint64_t)g->n);
+    if (cap > g->slot_epoch_cap) cap = g->slot_epoch_cap;
+    if (cap > (1ull << 24)) cap = 1ull << 24;
+    if (cap == 0) return fail(g, LAP_ERR_OOM, "workspace smaller than one tree");
+    *c = n_samples < cap ? n_samples : cap;
+    p.count = (uint32_t)*c;
+    p.slots = *c;
+    p.ws = g->ws;
+    p.slot_epoch = g->d_slot_epoch;
+    p.flags = LAP_SAMPLE_ONE_PER_LANE | LAP_SAMPLE_WILSON_ONLY;
+    LAP_CUDA(g, lap_launch_sample(p, g->stream));
+    t->trees = reinterpret_cast<const uint32_t *>(g->ws);
+    t->tree_stride = 2;
+    return LAP_OK;
+}
+
 lap_status lap_spantree_sample(lap_graph *g, uint64_t n_samples, uint64_t seed)
 {
     lap_status s = check_sticky(g);
@@ -1012,40 +1078,30 @@ lap_status lap_spantree_sample(lap_graph *g, uint64_t n_samples, uint64_t seed)
     if (n_samples == 0) return LAP_OK;
     if ((s = resolve_pending(g)) != LAP_OK) return s;      // the workspace is about to be reused
     if ((s = spantree_prepare(g)) != LAP_OK) return s;
-    if ((s = ensure_workspace(g, LAP_KERNEL_WIDE)) != LAP_OK) return s;
+    if (!g->ws && (s = ensure_workspace(g, LAP_KERNEL_WIDE)) != LAP_OK) return s;
     g->st_seed = seed;
     g->st_seed_set = true;
-    const uint64_t per_tree = 8ull * (uint64_t)g->n;
-    uint64_t cap = g->ws_bytes / per_tree;
-    if (cap > g->slot_epoch_cap) cap = g->slot_epoch_cap;
-    if (cap > (1ull << 24)) cap = 1ull << 24;
-    if (cap == 0) return fail(g, LAP_ERR_OOM, "workspace smaller than one tree");
     const uint64_t limit = g->step_limit ? g->step_limit : default_step_limit(g->n);
     for (uint64_t done = 0; done < n_samples;) {
-        const uint64_t c = n_samples - done < cap ? n_samples - done : cap;
         LapSampleLaunch p;
         memset(&p, 0, sizeof(p));
         p.g = LapDevGraph{g->d_rowinfo, g->d_col, g->n, g->arcs};
         p.root = g->root;
         p.seed = seed;
         p.first = (uint32_t)(g->st_cursor + done);
-        p.count = (uint32_t)c;
-        p.slots = c;
-        p.ws = g->ws;
-        p.slot_epoch = g->d_slot_epoch;
         p.rep1 = g->d_st_rep1;
         p.cnt2 = g->d_st_rep1;
         p.acc = g->d_st_acc;
         p.step_limit = limit;
         p.block = g->block_opt;
         p.num_sms = g->num_sms;
-        p.flags = LAP_SAMPLE_ONE_PER_LANE | LAP_SAMPLE_WILSON_ONLY;
-        LAP_CUDA(g, lap_launch_sample(p, g->stream));
         LapSpanTreeLaunch t;
         memset(&t, 0, sizeof(t));
+        uint64_t c = 0;
+        if ((s = spantree_block(g, p, n_samples - done, &c, &t)) != LAP_OK) return s;
+        if (c == 0 && (s = spantree_wide(g, p, n_samples - done, &c, &t)) != LAP_OK) return s;
         t.rowinfo = g->d_rowinfo;
         t.bpar = g->d_bpar;
-        t.trees = reinterpret_cast<const unsigned long long *>(g->ws);
         t.n = g->n;
         t.root = g->root;
         t.count = (uint32_t)c;
@@ -1061,14 +1117,7 @@ lap_status lap_spantree_sample(lap_graph *g, uint64_t n_samples, uint64_t seed)
     LapDevAcc h;
     LAP_CUDA(g, cudaMemcpyAsync(&h, g->d_st_acc, sizeof(h), cudaMemcpyDeviceToHost, g->stream));
     LAP_CUDA(g, cudaStreamSynchronize(g->stream));
-    if (h.status & LAP_DEV_STEP_LIMIT) {
-        g->sticky = LAP_ERR_STEP_LIMIT;
-        return fail(g, LAP_ERR_STEP_LIMIT, "a Wilson run exceeded the per-sample step budget (LAP_OPT_STEP_LIMIT)");
-    }
-    if (h.status) {
-        g->sticky = LAP_ERR_CUDA;
-        return fail(g, LAP_ERR_CUDA, "internal error in the SpanTree kernels (status " + std::to_string(h.status) + ")");
-    }
+    if (h.status) return spantree_failed(g, h.status);
     g->st_cursor += n_samples;
     g->st_omega += n_samples;
     return LAP_OK;

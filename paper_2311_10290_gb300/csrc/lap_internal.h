@@ -99,14 +99,16 @@ struct LapSampleLaunch {
     unsigned long long *cv_a2;
     unsigned long long *cv_p2;
     double *m2_out;              // optional [count]: per-sample M2 (with y1_out)
-    uint32_t flags;              // wide kernel: LAP_SAMPLE_* below
+    uint32_t *tree_out;          // block kernel, optional [count * n]: Next of every node (undefined at the
+                                 // root and in withdrawn samples)
+    uint32_t flags;              // LAP_SAMPLE_* below
     uint32_t ustart;             // 0: the first absorbed walk (or path) starts at a uniform draw
                                  // (Alg. 2); s + 1: it starts at node s (single-source rows of L_v^{-1})
 };
 enum : uint32_t {
-    LAP_SAMPLE_ONE_PER_LANE = 1u,   // lane j runs exactly sample first + j (j < count), so its
+    LAP_SAMPLE_ONE_PER_LANE = 1u,   // wide kernel: lane j runs exactly sample first + j (j < count), so its
                                     // slot ends holding that sample's tree (Next of every node)
-    LAP_SAMPLE_WILSON_ONLY = 2u,    // skip the two absorbed walks (no cnt2 passes, Y2 and M2 not written)
+    LAP_SAMPLE_WILSON_ONLY = 2u,    // wide and block kernel: skip the two absorbed walks (no cnt2 passes, Y2 and M2 not written)
 };
 cudaError_t lap_launch_sample(const LapSampleLaunch &p, cudaStream_t st);
 // sampler_compact.cu
@@ -255,7 +257,8 @@ cudaError_t lap_launch_finalize_batch(const LapBatchGraph *graphs, int32_t n_gra
 struct LapSpanTreeLaunch {
     const int2 *rowinfo;
     const int32_t *bpar;                 // [n] BFS parent (-1 at the root)
-    const unsigned long long *trees;     // count slots of n 8-byte Wilson states (low 32 bits: Next)
+    const uint32_t *trees;               // Next of node u in tree j: trees[(j * n + u) * tree_stride]
+    uint32_t tree_stride;
     int32_t n;
     int32_t root;
     uint32_t count;                      // trees in this launch

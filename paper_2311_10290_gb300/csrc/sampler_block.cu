@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(1024, 1) lewalk_block_kernel(LapSampleLaunch p
     const uint32_t wilson = blockDim.x - 32u;            // Wilson threads; the last warp runs the walks
     const Graph<PACK> g{p.g.rowinfo, p.g.col, b.arcs, b.bw, b.bo, policy_evict_last()};
     if (threadIdx.x >= wilson) {
-        walk_tasks<CV, PACK>(p, b, g);
+        if (!(p.flags & LAP_SAMPLE_WILSON_ONLY)) walk_tasks<CV, PACK>(p, b, g);
         return;
     }
     const uint32_t n = (uint32_t)p.g.n, v = (uint32_t)p.root;
@@ -932,12 +932,21 @@ __global__ void __launch_bounds__(1024, 1) lewalk_block_kernel(LapSampleLaunch p
             }
             if (j == 0) {
                 const unsigned int ix = atomicAdd(&p.acc->ovf_count, 1u);
-                if (ix < p.count) p.ovf_ids[ix] = i;
+                if (p.ovf_ids && ix < p.count) p.ovf_ids[ix] = i;
             }
         } else if (j == 0) {
             const unsigned long long y1 = (unsigned long long)(n - 1u) + lds64(ctl + cPops);
             acc1 += y1;
             if (p.y1_out) p.y1_out[q] = y1;
+        }
+        if (p.tree_out && !st) {
+            // The tree: every node's current arrow.
+            uint32_t *out = p.tree_out + (uint64_t)q * n;
+            for (uint32_t x = j; x < n; x += wilson) {
+                uint32_t o, dg;
+                g.row(x, o, dg);
+                out[x] = g.target(g.arc(o + below32(lap::philox_r64(x, d.k(x), i, 0u, key0, key1), dg)));
+            }
         }
         group_sync();
         if (bad) break;

@@ -7,8 +7,7 @@
 // nodes is a chain of a few thousand dependent steps that more walkers do not
 // shorten (its walks hit the root late and meet each other before), so what
 // counts is the time of one step: about 300 cycles here, where the 1-byte
-// kernel waits for three L2 or DRAM accesses per step.  Erdos-Renyi, 1000 nodes,
-// 10000 samples: 9.4 -> 4.4 ms.
+// kernel waits for three L2 or DRAM accesses per step.
 //
 // State per sample: one tree bit, one path bit and one byte of draws per node,
 // laid out word by word across the warp's lanes (word w of lane l at w * 32 + l),

@@ -18,61 +18,29 @@
 // (Alg. 1 prints the subtree test the other way round and applies it to x2
 // as well; the text and the flow argument fix the reading used here.)
 //
-// The trees come from the 8-byte Wilson kernel run with one sample per lane
-// (its slot ends holding Next of every node).  One CTA processes one tree:
-// children lists by counting sort, the tree's levels from v, subtree sizes
-// and degree sums bottom-up, preorder intervals top-down, then the BFS-path
-// sums for every node.  All per-node sums are integers, so accumulating them
+// The trees come from the block kernel (sampler_block.cu: a node's current arrow
+// when its sample is complete), or, where the workspace does not hold that, from
+// the 8-byte Wilson kernel run with one sample per lane (its slot ends holding
+// Next of every node; 512 trees of 50,000 nodes are 512 lanes on 152 SMs: 247 ms
+// against 3.5).  One CTA processes one tree:
+// subtree sizes and degree sums from the leaves up, without levels, preorder
+// intervals by pointer jumping, then the BFS-path sums for every node.  (With
+// children lists and a barrier per level of the tree, twice, 512 trees of 50,000
+// nodes took 11.9 ms; now 5.9.)  All per-node sums are integers, so accumulating them
 // over trees with atomics is exact and deterministic.
 #include "lap_internal.h"
 
 namespace {
 
-constexpr int kTB = 512;          // threads per tree CTA
+constexpr int kTB = 1024;         // threads per tree CTA
 constexpr int kFB = 256;          // finalize block
 constexpr int kParts = 1024;      // finalize partial sums (fixed order)
 
-__device__ __forceinline__ int32_t parent_of(const unsigned long long *tree, int32_t u)
-{
-    return (int32_t)(uint32_t)tree[u];
-}
-
-// Exclusive prefix sum of in[0..n) into out[0..n] (out[n] = total), by one CTA.
-__device__ void block_exclusive_scan(const int32_t *in, int32_t *out, int32_t n)
-{
-    __shared__ int32_t warp_tot[kTB / 32];
-    __shared__ int32_t carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int32_t base = 0; base < n; base += kTB) {
-        const int32_t idx = base + (int32_t)threadIdx.x;
-        const int32_t x = idx < n ? in[idx] : 0;
-        int32_t incl = x;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        if (lane == 31) warp_tot[wid] = incl;
-        __syncthreads();
-        if (wid == 0) {
-            int32_t t = lane < kTB / 32 ? warp_tot[lane] : 0;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int32_t y = __shfl_up_sync(0xFFFFFFFFu, t, o);
-                if (lane >= o) t += y;
-            }
-            if (lane < kTB / 32) warp_tot[lane] = t;     // inclusive over warps
-        }
-        __syncthreads();
-        const int32_t before = carry + (wid ? warp_tot[wid - 1] : 0);
-        if (idx < n) out[idx] = before + incl - x;
-        __syncthreads();
-        if (threadIdx.x == 0) carry += warp_tot[kTB / 32 - 1];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[n] = carry;
-    __syncthreads();
-}
+struct Tree {
+    const uint32_t *next;
+    uint32_t stride;
+};
+__device__ __forceinline__ int32_t parent_of(const Tree &t, int32_t u) { return (int32_t)t.next[(uint64_t)u * t.stride]; }
 
 __global__ void bfs_parent_kernel(const int2 *__restrict__ rowinfo, const int32_t *__restrict__ col,
                                   const int32_t *__restrict__ hops, int32_t n, int32_t root, int32_t *bpar,
@@ -96,22 +64,17 @@ __global__ void __launch_bounds__(kTB) spantree_tree_kernel(LapSpanTreeLaunch p)
 {
     const int32_t n = p.n, v = p.root;
     long long *dsum = reinterpret_cast<long long *>(p.scratch + (uint64_t)blockIdx.x * p.scratch_ints);
-    int32_t *cnt = reinterpret_cast<int32_t *>(dsum + n);
-    int32_t *off = cnt + n;             // n + 1
-    int32_t *child = off + n + 1;       // n
-    int32_t *queue = child + n;         // n
-    int32_t *lstart = queue + n;        // n + 2
-    int32_t *size = lstart + n + 2;     // n
-    int32_t *pre = size + n;            // n
-    __shared__ int32_t tail;
-    __shared__ int32_t levels;
+    int2 *up = reinterpret_cast<int2 *>(dsum + n);      // {preorder distance, ancestor}
+    int32_t *size = reinterpret_cast<int32_t *>(up + n);
+    int32_t *kids = size + n;                           // children
+    int32_t *seen = kids + n;                           // children whose subtree is complete
     const int32_t tid = (int32_t)threadIdx.x;
 
     for (uint32_t j = blockIdx.x; j < p.count; j += gridDim.x) {
-        const unsigned long long *T = p.trees + (uint64_t)j * (uint64_t)n;
-        // Children lists of T (counting sort by parent).
+        const Tree T{p.trees + (uint64_t)j * (uint64_t)n * p.tree_stride, p.tree_stride};
         for (int32_t u = tid; u < n; u += kTB) {
-            cnt[u] = 0;
+            kids[u] = 0;
+            seen[u] = 0;
             size[u] = 1;
             dsum[u] = p.rowinfo[u].y;
         }
@@ -120,77 +83,52 @@ __global__ void __launch_bounds__(kTB) spantree_tree_kernel(LapSpanTreeLaunch p)
             if (u == v) continue;
             const int32_t a = parent_of(T, u);
             if ((uint32_t)a >= (uint32_t)n) { atomicOr(p.status, LAP_DEV_BAD_INDEX); continue; }
-            atomicAdd(&cnt[a], 1);
+            atomicAdd(&kids[a], 1);
         }
         __syncthreads();
-        block_exclusive_scan(cnt, off, n);
-        for (int32_t u = tid; u < n; u += kTB) cnt[u] = 0;
-        __syncthreads();
+        // Subtree sizes and degree sums: from every leaf upwards, on by the last
+        // child to arrive at a node.  What a node's size was when its child's was
+        // added is the child's preorder distance below it.
         for (int32_t u = tid; u < n; u += kTB) {
-            if (u == v) continue;
-            const int32_t a = parent_of(T, u);
-            if ((uint32_t)a >= (uint32_t)n) continue;
-            child[off[a] + atomicAdd(&cnt[a], 1)] = u;
-        }
-        __syncthreads();
-        // Levels of T from v (queue holds the nodes level by level).
-        if (tid == 0) {
-            queue[0] = v;
-            lstart[0] = 0;
-            lstart[1] = 1;
-            tail = 1;
-            levels = 1;
-        }
-        __syncthreads();
-        for (int32_t L = 0;; ++L) {
-            const int32_t a = lstart[L], b = lstart[L + 1];
-            if (a == b || b >= n) break;
-            for (int32_t idx = a + tid; idx < b; idx += kTB) {
-                const int32_t u = queue[idx];
-                for (int32_t c = off[u]; c < off[u + 1]; ++c) {
-                    const int32_t pos = atomicAdd(&tail, 1);
-                    if (pos < n) queue[pos] = child[c];
-                }
+            if (kids[u] != 0 || u == v) continue;
+            for (int32_t x = u;;) {
+                const int32_t a = parent_of(T, x);
+                if ((uint32_t)a >= (uint32_t)n) break;
+                const int32_t before = atomicAdd(&size[a], __ldcg(&size[x]));
+                atomicAdd(reinterpret_cast<unsigned long long *>(&dsum[a]), (unsigned long long)__ldcg(&dsum[x]));
+                up[x] = make_int2(before, a);
+                if (a == v) break;
+                __threadfence_block();
+                if (atomicAdd(&seen[a], 1) + 1 != kids[a]) break;
+                __threadfence_block();
+                x = a;
             }
-            __syncthreads();
-            if (tid == 0) {
-                lstart[L + 2] = tail < n ? tail : n;
-                levels = L + 2;
-            }
-            __syncthreads();
         }
-        if (tid == 0 && tail != n) atomicOr(p.status, LAP_DEV_BAD_INDEX);   // not a spanning tree
+        if (tid == 0) up[v] = make_int2(0, v);
         __syncthreads();
-        const int32_t nl = levels;       // levels 0 .. nl-1 hold nodes
-        // Subtree sizes and degree sums, deepest level first.
-        for (int32_t L = nl - 1; L >= 1; --L) {
-            for (int32_t idx = lstart[L] + tid; idx < lstart[L + 1]; idx += kTB) {
-                const int32_t u = queue[idx];
-                const int32_t a = parent_of(T, u);
-                atomicAdd(&size[a], size[u]);
-                atomicAdd(reinterpret_cast<unsigned long long *>(&dsum[a]), (unsigned long long)dsum[u]);
-            }
+        if (__ldcg(&size[v]) != n) {                        // not a spanning tree
+            if (tid == 0) atomicOr(p.status, LAP_DEV_BAD_INDEX);
             __syncthreads();
+            continue;
         }
-        // Preorder intervals: u's subtree is [pre[u], pre[u] + size[u]).
-        if (tid == 0) pre[v] = 0;
-        __syncthreads();
-        for (int32_t L = 0; L < nl - 1; ++L) {
-            for (int32_t idx = lstart[L] + tid; idx < lstart[L + 1]; idx += kTB) {
-                const int32_t u = queue[idx];
-                int32_t next_pre = pre[u] + 1;
-                for (int32_t c = off[u]; c < off[u + 1]; ++c) {
-                    const int32_t w = child[c];
-                    pre[w] = next_pre;
-                    next_pre += size[w];
-                }
+        // Preorder numbers, the sums of the distances up to v, by pointer jumping
+        // in place: whichever pair of the ancestor is read, its distance is that to
+        // the ancestor it names.  u's subtree is [pre[u], pre[u] + size[u]).
+        for (int32_t round = 0; round < 32; ++round) {
+            bool more = false;
+            for (int32_t u = tid; u < n; u += kTB) {
+                const int2 a = up[u];
+                if (a.y == v) continue;
+                const unsigned long long w = __ldcg(reinterpret_cast<const unsigned long long *>(up + a.y));
+                up[u] = make_int2(a.x + (int32_t)(uint32_t)w, (int32_t)(w >> 32));
+                more = more || (int32_t)(w >> 32) != v;
             }
-            __syncthreads();
+            if (!__syncthreads_or(more)) break;
         }
         // The sums along every node's BFS path.
         for (int32_t u = tid; u < n; u += kTB) {
             long long x1 = 0, x2 = 0, x2d = 0;
-            const int32_t pu = pre[u];
+            const int32_t pu = up[u].x;
             int32_t e1 = u;
             for (int32_t guard = 0; e1 != v && guard < n; ++guard) {
                 const int32_t e2 = p.bpar[e1];
@@ -198,11 +136,11 @@ __global__ void __launch_bounds__(kTB) spantree_tree_kernel(LapSpanTreeLaunch p)
                 if (parent_of(T, e1) == e2) {
                     x2 += size[e1];
                     x2d += dsum[e1];
-                    if (pre[e1] <= pu && pu < pre[e1] + size[e1]) ++x1;
+                    if (up[e1].x <= pu && pu < up[e1].x + size[e1]) ++x1;
                 } else if (e2 != v && parent_of(T, e2) == e1) {
                     x2 -= size[e2];
                     x2d -= dsum[e2];
-                    if (pre[e2] <= pu && pu < pre[e2] + size[e2]) --x1;
+                    if (up[e2].x <= pu && pu < up[e2].x + size[e2]) --x1;
                 }
                 e1 = e2;
             }
@@ -299,9 +237,8 @@ cudaError_t lap_launch_bfs_parent(const int2 *rowinfo, const int32_t *col, const
 
 uint64_t lap_spantree_scratch_ints(int32_t n)
 {
-    // dsum (2n ints) + cnt n + off n+1 + child n + queue n + lstart n+2 + size n + pre n, rounded to even.
-    const uint64_t ints = 2ull * (uint64_t)n + 7ull * (uint64_t)n + 3ull;
-    return (ints + 1ull) & ~1ull;
+    // dsum (2 n), up (2 n), size, kids, seen, rounded up to whole 64-bit words.
+    return (7ull * (uint64_t)n + 1ull) & ~1ull;
 }
 
 int lap_spantree_block() { return kTB; }
