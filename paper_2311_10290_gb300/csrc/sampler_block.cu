@@ -19,7 +19,7 @@
 //     for each node).  If a k has changed, another walker has popped one of the
 //     nodes: the walk goes on from the closing node.
 // Two-node cycles (nearly all of them) take the lock bits of their two nodes,
-// lowest id first; longer ones take the sample's exclusive flag, which keeps
+// lowest lock first; longer ones take the sample's exclusive flag, which keeps
 // two-node pops out, and are checked and popped by all lanes of the warp.
 // A stale path entry can only fail such a check, never count; nodes walked by
 // two walkers cost time and no counts.  Locks are held across straight-line
@@ -206,7 +206,10 @@ template <bool CV>
 __device__ __forceinline__ uint32_t pop_pair(const Draws &d, uint32_t ctl, uint32_t u, uint32_t ku, uint32_t w,
                                              uint32_t kw, const LapSampleLaunch &p, unsigned &status)
 {
-    const uint32_t a = u < w ? u : w, b = u < w ? w : u;
+    // By lock index: in any other order, two pairs whose locks coincide crosswise
+    // could fail each other again and again.
+    const bool first = (u & d.lmask) < (w & d.lmask);
+    const uint32_t a = first ? u : w, b = first ? w : u;
     atoms_add(ctl + cInflight, 1u);
     __threadfence_block();
     bool ok = !lds(ctl + cExcl) && d.try_lock(a);

@@ -2,7 +2,8 @@
 automatic calls take on graphs above the small-graph kernel's range, at the
 sizes where it can go wrong: node counts around a word of tree bits, samples
 around the number in flight, a workspace too small for the early phase or for
-more than one sample, loop-included paths, control-variate sums, and cycles
+more than one sample, long first walks whose tables fit a part of the call only,
+loop-included paths, control-variate sums, and cycles
 longer than the bookkeeping's short forms.  Integers are bit-exact with the
 sequential oracle."""
 import numpy as np
@@ -15,7 +16,8 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 import oracle.cv as CV  # noqa: E402
-from paper_2311_10290_gb300.lap import LAP_OPT_PATHS, LAP_OPT_SLOTS, LAP_STAT_LAST_KERNEL, LapGraph  # noqa: E402
+from paper_2311_10290_gb300.lap import (LAP_OPT_PATHS, LAP_OPT_SLOTS, LAP_STAT_FALLBACKS, LAP_STAT_LAST_KERNEL,  # noqa: E402
+                                        LapGraph)
 
 
 def grid(k):
@@ -23,6 +25,13 @@ def grid(k):
     x = np.arange(k * k).reshape(k, k)
     e = np.concatenate([np.stack([x[:, :-1].ravel(), x[:, 1:].ravel()], 1), np.stack([x[:-1].ravel(), x[1:].ravel()], 1)])
     return I.from_edges(k * k, e)
+
+
+def crossed_pairs():
+    """A star with its leaves paired 8192 ids apart but for the lowest bit: the locks
+    (13 low id bits) of neighbouring pairs coincide crosswise."""
+    i, leaf = np.arange(2, 8192), np.arange(1, 16384)
+    return I.from_edges(16384, np.concatenate([np.stack([i, 8192 + (i ^ 1)], 1), np.stack([0 * leaf, leaf], 1)]))
 
 
 CASES = [("word_minus_1", lambda: I.ba(4127, 3, seed=1), 40, {}),
@@ -35,7 +44,9 @@ CASES = [("word_minus_1", lambda: I.ba(4127, 3, seed=1), 40, {}),
          ("paths", lambda: I.ba(6000, 3, seed=7), 100, dict(paths=True, trace=True)),
          ("hubs", lambda: I.rmat(14, 8, seed=8), 64, dict(trace=True)),
          ("star", lambda: I.star(5000), 64, dict(root=17)),
-         ("grid", lambda: grid(66), 24, dict(root=0))]
+         ("grid", lambda: grid(66), 24, dict(root=0)),
+         ("parts", lambda: I.er(12000, 6 / 12000, seed=9), 300, dict(ws=24 << 20, trace=True)),
+         ("crossed_pairs", crossed_pairs, 200, dict(no_reruns=True))]
 
 
 @pytest.mark.parametrize("cv", [False, True], ids=["plain", "cv"])
@@ -62,6 +73,7 @@ def test_block_kernel_matches_oracle(maker, omega, o, cv):
                 G.sample(part, 41)
         c1, c2, s = G.counts()
         assert G.stat(LAP_STAT_LAST_KERNEL) == 3
+        assert not o.get("no_reruns") or G.stat(LAP_STAT_FALLBACKS) == 0
         sums = G.cv_sums() if cv else None
     finally:
         G.close()
