@@ -47,6 +47,9 @@ void free_all(lap_graph *g)
     cudaFree(g->d_rowinfo);
     cudaFree(g->d_arcs);
     cudaFree(g->d_hubs);
+    if (g->side) cudaStreamDestroy(g->side);
+    if (g->fork) cudaEventDestroy(g->fork);
+    if (g->joined) cudaEventDestroy(g->joined);
     cudaFree(g->d_hops);
     cudaFree(g->d_rep1);
     cudaFree(g->d_cnt2);
@@ -251,7 +254,7 @@ bool choose_cta(const lap_graph *g, uint64_t n_samples, LapCtaPlan *pl)
 {
     if (g->walkers || g->compact_disabled || !g->ws) return false;
     if (g->kernel_opt != 0 && g->kernel_opt != LAP_KERNEL_GROUP) return false;
-    return lap_cta_plan(g->n, g->arcs, n_samples, g->slots_opt, g->ws_bytes, g->num_sms, g->paths_opt != 0, g->cv1 || g->cv2,
+    return lap_cta_plan(g->n, g->arcs, g->root_degree, g->max_degree, n_samples, g->slots_opt, g->ws_bytes, g->num_sms, g->paths_opt != 0, g->cv1 || g->cv2,
                         g->d_arcs != nullptr, pl);
 }
 
@@ -271,7 +274,14 @@ lap_status launch_cta(lap_graph *g, LapSampleLaunch &p, LapCtaPlan &pl)
     g->tag_next += p.count;
     LAP_CUDA(g, cudaMemsetAsync(&g->d_acc->claim, 0, sizeof(unsigned int), g->stream));
     LAP_CUDA(g, cudaMemsetAsync(&g->d_acc->walk_claim, 0, sizeof(unsigned int), g->stream));
-    const cudaError_t e = lap_launch_cta(p, pl, g->ws, g->d_arcs, tag, g->stream);
+    lap_cta_bind(p, pl, g->ws, g->d_arcs, tag);
+    LAP_CUDA(g, cudaEventRecord(g->fork, g->stream));
+    LAP_CUDA(g, cudaStreamWaitEvent(g->side, g->fork, 0));
+    cudaError_t e = lap_launch_cta_walks(p, pl, g->side);
+    if (e == cudaSuccess) e = lap_launch_cta_wilson(p, pl, g->stream);
+    const cudaError_t f = cudaEventRecord(g->joined, g->side);
+    if (e == cudaSuccess) e = f;
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(g->stream, g->joined, 0);
     if (e != cudaSuccess) return cuda_fail(g, e, "sampler launch (kernel 3)");
     return LAP_OK;
 }
@@ -411,6 +421,9 @@ lap_status lap_graph_create(int32_t n, const int32_t *row_ptr, const int32_t *co
         return bad;
     }
     e = lap_launch_rowinfo(g->d_row_ptr, n, g->d_rowinfo, g->stream);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&g->side, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g->fork, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g->joined, cudaEventDisableTiming);
     // Hubs, in id order (the row kernels' sums keep one order).
     unsigned int hub_count = 0;
     if (e == cudaSuccess && dalloc(&g->d_hubs, (size_t)(last / LAP_HUB_DEGREE) + 1) != cudaSuccess) {
@@ -433,6 +446,12 @@ lap_status lap_graph_create(int32_t n, const int32_t *row_ptr, const int32_t *co
         if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
     }
     g->hubs = LapHubs{g->d_hubs, (int32_t)hub_count};
+    unsigned long long top = 0;
+    if (e == cudaSuccess) e = cudaMemsetAsync(g->d_red, 0, sizeof(top), g->stream);
+    if (e == cudaSuccess) e = lap_launch_argmax_degree(g->d_rowinfo, n, reinterpret_cast<unsigned long long *>(g->d_red), g->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&top, g->d_red, sizeof(top), cudaMemcpyDeviceToHost, g->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
+    g->max_degree = (int32_t)(top >> 32);
     // Packed arcs where they stay in L2 (an allocation that fails leaves the
     // plain columns).
     if (e == cudaSuccess && n <= (1 << 21) && 8ull * (uint64_t)last <= kL2Graph) {
@@ -579,6 +598,8 @@ lap_status lap_set_root(lap_graph *g, int32_t v, int32_t *root_out)
         LAP_CUDA(g, cudaStreamSynchronize(g->stream));
         v = (int32_t)(0xFFFFFFFFu - (uint32_t)(h & 0xFFFFFFFFull));
     }
+    int2 record = make_int2(0, 0);
+    LAP_CUDA(g, cudaMemcpyAsync(&record, g->d_rowinfo + v, sizeof(record), cudaMemcpyDeviceToHost, g->stream));
     // Breadth-first search from v: connectivity check and hop distances.
     int64_t reached = 0;
     LAP_CUDA(g, lap_run_bfs(g->d_rowinfo, g->d_col, g->n, g->hubs, v, g->d_hops, reinterpret_cast<unsigned int *>(g->d_red),
@@ -612,6 +633,7 @@ lap_status lap_set_root(lap_graph *g, int32_t v, int32_t *root_out)
     g->compact_disabled = false;
     g->fallbacks = 0;
     g->root = v;
+    g->root_degree = record.y;
     g->seed_set = false;
     g->omega = 0;
     g->cursor = 0;
@@ -1024,7 +1046,7 @@ static lap_status spantree_block(lap_graph *g, LapSampleLaunch &p, uint64_t n_sa
     if (m > n_samples) m = n_samples;
     if (m > (1ull << 24)) m = 1ull << 24;
     LapCtaPlan pl;
-    if (m == 0 || !lap_block_plan(g->n, m, g->slots_opt, half, g->num_sms, false, false, g->d_arcs != nullptr, &pl.block))
+    if (m == 0 || !lap_block_plan(g->n, g->arcs, g->root_degree, g->max_degree, m, g->slots_opt, half, g->num_sms, false, false, g->d_arcs != nullptr, &pl.block))
         return LAP_OK;
     g->last_kernel = LAP_KERNEL_GROUP;
     g->ws_zeroed = false;
@@ -1033,9 +1055,9 @@ static lap_status spantree_block(lap_graph *g, LapSampleLaunch &p, uint64_t n_sa
     LAP_CUDA(g, cudaMemsetAsync(&g->d_st_acc->claim, 0, sizeof(unsigned int), g->stream));
     LAP_CUDA(g, cudaMemsetAsync(&g->d_st_acc->ovf_count, 0, sizeof(unsigned int), g->stream));
     p.count = (uint32_t)m;
-    p.flags = LAP_SAMPLE_WILSON_ONLY;
     p.tree_out = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(g->ws) + half);
-    LAP_CUDA(g, lap_launch_cta(p, pl, g->ws, g->d_arcs, 0u, g->stream));
+    lap_cta_bind(p, pl, g->ws, g->d_arcs, 0u);
+    LAP_CUDA(g, lap_launch_cta_wilson(p, pl, g->stream));
     LapDevAcc h;
     LAP_CUDA(g, cudaMemcpyAsync(&h, g->d_st_acc, sizeof(h), cudaMemcpyDeviceToHost, g->stream));
     LAP_CUDA(g, cudaStreamSynchronize(g->stream));

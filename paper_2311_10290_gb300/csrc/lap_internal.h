@@ -108,7 +108,7 @@ struct LapSampleLaunch {
 enum : uint32_t {
     LAP_SAMPLE_ONE_PER_LANE = 1u,   // wide kernel: lane j runs exactly sample first + j (j < count), so its
                                     // slot ends holding that sample's tree (Next of every node)
-    LAP_SAMPLE_WILSON_ONLY = 2u,    // wide and block kernel: skip the two absorbed walks (no cnt2 passes, Y2 and M2 not written)
+    LAP_SAMPLE_WILSON_ONLY = 2u,    // wide kernel: skip the two absorbed walks (no cnt2 passes, Y2 and M2 not written)
 };
 cudaError_t lap_launch_sample(const LapSampleLaunch &p, cudaStream_t st);
 // sampler_compact.cu
@@ -145,11 +145,14 @@ struct LapBlockLaunch {
     uint32_t early_nodes, early_budget;       // tree size and step budget at which it ends
     uint32_t early_entries, early_log2;       // table entries of a sample
     uint32_t early_cap;                       // path entries of a sample
+    uint32_t part;                            // samples of the call that are run at a time
+    uint32_t ovf_cap;                         // entries of LapSampleLaunch::ovf_ids
     uint32_t *early, *early_stacks, *early_pops;
 };
 struct LapBlockPlan {
     LapBlockLaunch b = {};
-    int threads = 0;                  // Wilson threads per CTA (one more warp runs the absorbed walks)
+    int threads = 0;                  // per CTA
+    uint64_t walk_ctas = 0;           // CTAs (of a warp) for the absorbed walks
     uint64_t slots = 0, smem = 0;     // CTAs (samples in flight), shared memory of each
     uint64_t words_bytes = 0;         // words and path words, zeroed when the layout grows
     uint64_t path_offset = 0, stack_offset = 0, sweep_offset = 0, early_offset = 0;
@@ -157,14 +160,15 @@ struct LapBlockPlan {
 void lap_pack_bits(int32_t n, int64_t arcs, uint32_t *bw, uint32_t *bo);
 cudaError_t lap_launch_pack_arcs(const int2 *rowinfo, const int32_t *col, int32_t n, int64_t arcs,
                                  unsigned long long *out, cudaStream_t st);
-bool lap_block_plan(int32_t n, uint64_t count, uint64_t slots_opt, uint64_t ws_bytes, int num_sms, bool paths, bool cv,
+bool lap_block_plan(int32_t n, int64_t arcs, int32_t root_degree, int32_t max_degree, uint64_t count, uint64_t slots_opt, uint64_t ws_bytes, int num_sms, bool paths, bool cv,
                     bool pack, LapBlockPlan *out);
 cudaError_t lap_launch_sample_block(const LapSampleLaunch &p, const LapBlockPlan &pl, cudaStream_t st);
 
 // sampler_small.cu: a lane per sample, state and graph in shared memory
 struct LapSmallPlan {
     LapBlockLaunch b = {};            // arcs, path words, stacks, tags
-    int warps = 0;                    // per CTA (one more runs the absorbed walks)
+    int warps = 0;                    // per CTA
+    uint64_t walk_ctas = 0;           // CTAs (of a warp) for the absorbed walks
     uint32_t lanes = 0;               // lanes of a warp that take samples
     bool local = false;               // the graph is copied to shared memory
     uint64_t slots = 0, blocks = 0, smem = 0, words_bytes = 0, stack_offset = 0, many_offset = 0;
@@ -180,11 +184,14 @@ struct LapCtaPlan {
     LapSmallPlan lane;
     uint64_t words_bytes() const { return small ? lane.words_bytes : block.words_bytes; }
 };
-bool lap_cta_plan(int32_t n, int64_t arcs, uint64_t count, uint64_t slots_opt, uint64_t ws_bytes, int num_sms, bool paths,
+bool lap_cta_plan(int32_t n, int64_t arcs, int32_t root_degree, int32_t max_degree, uint64_t count, uint64_t slots_opt, uint64_t ws_bytes, int num_sms, bool paths,
                   bool cv, bool pack, LapCtaPlan *out);
-// ws: its first words_bytes() hold zeros, or words of this layout under other tags
-cudaError_t lap_launch_cta(LapSampleLaunch &p, LapCtaPlan &pl, void *ws, const unsigned long long *arcs, uint32_t tag_base,
-                           cudaStream_t st);
+// Fills in the plan's pointers: ws: its first words_bytes() hold zeros, or
+// words of this layout under other tags.
+void lap_cta_bind(LapSampleLaunch &p, LapCtaPlan &pl, void *ws, const unsigned long long *arcs, uint32_t tag_base);
+// The two parts of a launch; they share no state and may run side by side.
+cudaError_t lap_launch_cta_wilson(const LapSampleLaunch &p, const LapCtaPlan &pl, cudaStream_t st);
+cudaError_t lap_launch_cta_walks(const LapSampleLaunch &p, const LapCtaPlan &pl, cudaStream_t st);
 
 // ------------------------------------------------------------ batches
 // One graph of a batch (device descriptor).  Pointers index the batch's
@@ -381,6 +388,9 @@ struct lap_graph {
     bool ws_owned = false;
     bool ws_zeroed = false;
     unsigned long long *d_arcs = nullptr;   // packed arcs (lap_launch_pack_arcs) of graphs that keep them in L2
+    cudaStream_t side = nullptr;            // absorbed walks, beside the Wilson runs on `stream`
+    cudaEvent_t fork = nullptr, joined = nullptr;
+    int32_t root_degree = 0, max_degree = 0;
     uint64_t blk_clean = 0;                 // leading workspace bytes that hold only the block kernel's tagged words
     uint32_t tag_next = 0;                  // sample tags used since they were zeroed
 

@@ -1,7 +1,6 @@
 // Cycle-popping LEWalk sampler with the tree in shared memory: one CTA runs one
-// sample's Wilson LE_v run, and the CTA's last warp runs the absorbed walks of
-// Alg. 2 and Alg. 4 (walk_tasks.cuh).  Counts are those of the sequential run,
-// bit for bit.
+// sample's Wilson LE_v run.  Counts are those of the sequential run, bit for bit.
+// (The absorbed walks of Alg. 2 and Alg. 4 run beside it, sampler_cta.cu.)
 //
 // Why it is exact.  In the stack representation of Section 3.4 (Fig. 1) node
 // u's j-th draw is the Philox draw (u, j, i, 0); Wilson's run pops cycles of
@@ -55,9 +54,10 @@
 // memory) while few lanes have work, and instruction issue (about 130 per
 // step) when all have.  Against a lane per sample with byte counts in HBM
 // (sampler_compact.cu), sampling only: Barabasi-Albert, 10^5 nodes, 16384
-// samples 173 -> 78 ms; 10^6 nodes, 4096 samples 750 -> 219 ms; R-MAT of 31
+// samples 173 -> 75 ms; 10^6 nodes, 4096 samples 750 -> 203 ms; R-MAT of 31
 // million arcs, 2048 samples 312 -> 39 ms; 2 * 10^5 nodes with control variate and
-// paths, 2048 samples 196 -> 31 ms.
+// paths, 2048 samples 196 -> 27 ms; Erdos-Renyi, 10^5 nodes, 512 samples
+// 1288 -> 169 ms.
 #include <cmath>
 
 #include "walk_tasks.cuh"
@@ -257,8 +257,9 @@ __global__ void __launch_bounds__(128) lewalk_early_kernel(LapSampleLaunch p, La
     const uint32_t mask = b.early_entries - 1u, shift = 32u - b.early_log2;
     uint32_t off, deg, droot;
     g.row(v, off, droot);
-    // Expected steps: about 2m / d_v to the root, then a few per node.
-    const unsigned long long budget64 = 3ull * ((unsigned long long)p.g.arcs / droot) + 4ull * b.early_nodes;
+    // Expected steps: about 2m / d_v to the root, then a few per node.  A sample
+    // that is left without a tree costs the block kernel far more than a lane here.
+    const unsigned long long budget64 = 8ull * ((unsigned long long)p.g.arcs / droot) + 4ull * b.early_nodes;
     const uint32_t budget = budget64 > b.early_budget ? b.early_budget : (uint32_t)budget64;
     tbl[((v + 1u) * 2654435761u) >> shift] = (v + 1u) << kEKeyShift | kETree;
     uint32_t used = 1, done = 1, sp = 0, s = 0, u = 0, steps = 0, pops = 0;
@@ -328,18 +329,14 @@ __global__ void __launch_bounds__(128) lewalk_early_kernel(LapSampleLaunch p, La
     b.early_pops[q] = pops;
 }
 
-// One sample per CTA at a time; the last warp runs the absorbed walks.
+// One sample per CTA at a time.
 template <bool CV, bool PACK>
 __global__ void __launch_bounds__(1024, 1) lewalk_block_kernel(LapSampleLaunch p, LapBlockLaunch b)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t wilson = blockDim.x - 32u;            // Wilson threads; the last warp runs the walks
+    const uint32_t wilson = blockDim.x;
     const Graph<PACK> g{p.g.rowinfo, p.g.col, b.arcs, b.bw, b.bo, policy_evict_last()};
-    if (threadIdx.x >= wilson) {
-        if (!(p.flags & LAP_SAMPLE_WILSON_ONLY)) walk_tasks<CV, PACK>(p, b, g);
-        return;
-    }
     const uint32_t n = (uint32_t)p.g.n, v = (uint32_t)p.root;
     const uint32_t j = threadIdx.x;                      // walker index
     const uint64_t slot = blockIdx.x;
@@ -935,7 +932,7 @@ __global__ void __launch_bounds__(1024, 1) lewalk_block_kernel(LapSampleLaunch p
             }
             if (j == 0) {
                 const unsigned int ix = atomicAdd(&p.acc->ovf_count, 1u);
-                if (p.ovf_ids && ix < p.count) p.ovf_ids[ix] = i;
+                if (p.ovf_ids && ix < b.ovf_cap) p.ovf_ids[ix] = i;
             }
         } else if (j == 0) {
             const unsigned long long y1 = (unsigned long long)(n - 1u) + lds64(ctl + cPops);
@@ -1015,7 +1012,7 @@ cudaError_t lap_launch_pack_arcs(const int2 *rowinfo, const int32_t *col, int32_
 // shared memory and the workspace's layout (words, path words, stacks, sweep
 // arrays, early tables).  False: the graph's tree bits exceed an SM's shared
 // memory, or the workspace does not hold one sample.
-bool lap_block_plan(int32_t n, uint64_t count, uint64_t slots_opt, uint64_t ws_bytes, int num_sms, bool paths, bool cv,
+bool lap_block_plan(int32_t n, int64_t arcs, int32_t root_degree, int32_t max_degree, uint64_t count, uint64_t slots_opt, uint64_t ws_bytes, int num_sms, bool paths, bool cv,
                     bool pack, LapBlockPlan *out)
 {
     LapBlockPlan pl;
@@ -1052,23 +1049,51 @@ bool lap_block_plan(int32_t n, uint64_t count, uint64_t slots_opt, uint64_t ws_b
         return false;
     }
     if (resident < 1) return false;
+    // A warp of absorbed walks per CTA in flight, as counted for `resident`.
+    pl.walk_ctas = (uint64_t)resident * num_sms;
     uint64_t slots = want < (uint64_t)resident * num_sms ? want : (uint64_t)resident * num_sms;
-    // The workspace: shorter stacks first, then fewer samples in flight.
+    // Early phase: until about twice sqrt(8 / n) of the nodes are in the tree,
+    // where 32 walkers become useful.  A sample's table has four entries for each
+    // of them, and two for each node that a long first walk passes: it reaches
+    // the root after 2m / d_v steps on average, few beside a hub but 36,000 on an
+    // Erdos-Renyi graph of 100,000 nodes.
+    const uint64_t target = (uint64_t)(5.7 * sqrt((double)nn));
+    uint64_t pass = 4ull * ((uint64_t)arcs / (uint64_t)(root_degree > 0 ? root_degree : 1));
+    if (pass > nn) pass = nn;
+    // A hub is drawn about d / d_v times on the way to the root.  Where that is more
+    // than the tables' 9 bits count, samples reach the block kernel without a tree,
+    // and its walkers do not shorten the rest.  It is still the faster kernel for few
+    // samples (64 on a graph of 200,000 nodes, hub of degree 1823, rooted at degree 6:
+    // 1.3 s, a lane per sample 3.7 s), but runs them some 300 at a time, where the
+    // other kernels run all at once.
+    if (pass > 16ull * target && max_degree / 64 > root_degree && count > 4ull * num_sms) return false;
+    uint32_t lg = 10;
+    while ((1ull << lg) < 4ull * target || (1ull << lg) < 2ull * pass) ++lg;
+    b.early_log2 = lg;
+    b.early_entries = 1u << lg;
+    b.early_nodes = (uint32_t)target;
+    b.early_cap = 4096u;
+    b.early_budget = 1u << 22;
+    const uint64_t early_per = 4ull * b.early_entries + 4ull * b.early_cap + 4ull;
+    // The workspace: at most half for the early tables (none if no sample fits
+    // beside them); then shorter stacks, then fewer samples in flight.
     const uint64_t node_bytes = (8ull + 12ull) * nn;
     const uint64_t path_bytes = paths ? 8ull * nn : 0ull;       // one walk's departures, at least
     const uint64_t slack = 2048ull;
+    uint64_t reserve = early_per * count < ws_bytes / 2ull ? early_per * count : ws_bytes / 2ull;
     for (;;) {
         b.stack_entries = 32ull * b.cap_a + (uint64_t)(pl.threads - 32) * b.cap_b;
-        const uint64_t per = node_bytes + 8ull * b.stack_entries;
-        if (slots * per + path_bytes + slack <= ws_bytes) break;
+        const uint64_t per = node_bytes + 8ull * b.stack_entries, other = path_bytes + slack + reserve;
+        if (slots * per + other <= ws_bytes) break;
         if (b.cap_a > 4096u || b.cap_b > 64u) {
             // Not below 4096 (or 2 n): a cycle longer than every stack is never found.
             if (b.cap_a > 4096u) b.cap_a = 4096u;
             if (b.cap_b > 64u) b.cap_b /= 2u;
         } else {
-            const uint64_t fit = (ws_bytes > path_bytes + slack ? ws_bytes - path_bytes - slack : 0ull) / per;
-            if (fit == 0) return false;
-            slots = fit;
+            const uint64_t fit = (ws_bytes > other ? ws_bytes - other : 0ull) / per;
+            if (fit) slots = fit;
+            else if (reserve) reserve = 0;
+            else return false;
         }
     }
     pl.slots = slots;
@@ -1077,7 +1102,7 @@ bool lap_block_plan(int32_t n, uint64_t count, uint64_t slots_opt, uint64_t ws_b
         // At most half of the rest: the early tables need some too.
         b.path_lanes = (ws_bytes - fixed_bytes + path_bytes) / 2ull / path_bytes;
         if (b.path_lanes < 1ull) b.path_lanes = 1ull;
-        if (b.path_lanes > slots * 32ull) b.path_lanes = slots * 32ull;
+        if (b.path_lanes > pl.walk_ctas * 32ull) b.path_lanes = pl.walk_ctas * 32ull;
     }
     auto up = [](uint64_t x) { return (x + 255ull) & ~255ull; };
     pl.path_offset = slots * 8ull * nn;
@@ -1085,21 +1110,12 @@ bool lap_block_plan(int32_t n, uint64_t count, uint64_t slots_opt, uint64_t ws_b
     pl.stack_offset = up(pl.words_bytes);
     pl.sweep_offset = up(pl.stack_offset + 8ull * slots * b.stack_entries);
     pl.early_offset = up(pl.sweep_offset + 12ull * slots * nn);
-    // Early phase: until about twice sqrt(8 / n) of the nodes are in the tree,
-    // where 32 walkers become useful; a table of at least four times that many
-    // entries per sample, from what the workspace has left.
-    const uint64_t target = (uint64_t)(5.7 * sqrt((double)nn));
-    uint32_t lg = 10;
-    while ((1ull << lg) < 4ull * target) ++lg;
-    b.early_log2 = lg;
-    b.early_entries = 1u << lg;
-    b.early_nodes = (uint32_t)target;
-    b.early_cap = 4096u;
-    b.early_budget = 1u << 20;
-    const uint64_t per = 4ull * b.early_entries + 4ull * b.early_cap + 4ull;
-    uint64_t m = ws_bytes > pl.early_offset + 64ull ? (ws_bytes - pl.early_offset - 64ull) / per : 0ull;
+    // Early tables from what the workspace has left.
+    uint64_t m = ws_bytes > pl.early_offset + 64ull ? (ws_bytes - pl.early_offset - 64ull) / early_per : 0ull;
     if (m > count) m = count;
     b.early_count = (uint32_t)m;
+    // Where the first walk is long, a call whose tables do not fit runs in parts.
+    b.part = pass > 16ull * target && b.early_count > 0 && b.early_count < count ? b.early_count : (uint32_t)count;
     // Few samples per warp: a warp's lanes wait for each other.
     const uint64_t warps = 16ull * num_sms;
     const uint64_t l = (m + warps - 1) / warps;
@@ -1108,23 +1124,36 @@ bool lap_block_plan(int32_t n, uint64_t count, uint64_t slots_opt, uint64_t ws_b
     return true;
 }
 
-cudaError_t lap_launch_sample_block(const LapSampleLaunch &p, const LapBlockPlan &pl, cudaStream_t st)
+cudaError_t lap_launch_sample_block(const LapSampleLaunch &all, const LapBlockPlan &pl, cudaStream_t st)
 {
-    if (p.count == 0 || pl.slots == 0) return cudaSuccess;
-    const bool cv = p.cv_h1 || p.cv_h2, pack = pl.b.arcs != nullptr;
+    if (all.count == 0 || pl.slots == 0) return cudaSuccess;
+    const bool cv = all.cv_h1 || all.cv_h2, pack = pl.b.arcs != nullptr;
     const void *kernel = kernel_for(cv, pack);
-    if (pl.b.early_count) {
-        const cudaError_t e = cudaMemsetAsync(pl.b.early, 0, 4ull * pl.b.early_entries * pl.b.early_count, st);
+    for (uint32_t done = 0; done < all.count; done += pl.b.part) {
+        LapSampleLaunch p = all;
+        LapBlockLaunch b = pl.b;
+        p.first += done;
+        p.count = all.count - done < b.part ? all.count - done : b.part;
+        if (p.y1_out) p.y1_out += done;
+        if (p.tree_out) p.tree_out += (uint64_t)done * (uint64_t)p.g.n;
+        b.tag_base += done;
+        b.ovf_cap = all.count;
+        if (b.early_count > p.count) b.early_count = p.count;
+        cudaError_t e = done ? cudaMemsetAsync(&p.acc->claim, 0, sizeof(unsigned int), st) : cudaSuccess;
         if (e != cudaSuccess) return e;
-        const uint64_t per_block = 4ull * pl.b.early_lanes;
-        const unsigned blocks = (unsigned)((pl.b.early_count + per_block - 1) / per_block);
-        if (cv) pack ? launch_early<true, true>(p, pl.b, blocks, st) : launch_early<true, false>(p, pl.b, blocks, st);
-        else pack ? launch_early<false, true>(p, pl.b, blocks, st) : launch_early<false, false>(p, pl.b, blocks, st);
-        const cudaError_t f = cudaGetLastError();
-        if (f != cudaSuccess) return f;
+        if (b.early_count) {
+            e = cudaMemsetAsync(b.early, 0, 4ull * b.early_entries * b.early_count, st);
+            if (e != cudaSuccess) return e;
+            const uint64_t per_block = 4ull * b.early_lanes;
+            const unsigned blocks = (unsigned)((b.early_count + per_block - 1) / per_block);
+            if (cv) pack ? launch_early<true, true>(p, b, blocks, st) : launch_early<true, false>(p, b, blocks, st);
+            else pack ? launch_early<false, true>(p, b, blocks, st) : launch_early<false, false>(p, b, blocks, st);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
+        void *args[2] = {&p, &b};
+        const uint64_t ctas = pl.slots < p.count ? pl.slots : p.count;
+        e = cudaLaunchKernel(kernel, dim3((unsigned)ctas), dim3((unsigned)pl.threads), args, (size_t)pl.smem, st);
+        if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    void *args[2] = {const_cast<LapSampleLaunch *>(&p), const_cast<LapBlockLaunch *>(&pl.b)};
-    const cudaError_t e = cudaLaunchKernel(kernel, dim3((unsigned)pl.slots), dim3((unsigned)(pl.threads + 32)), args,
-                                           (size_t)pl.smem, st);
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return cudaSuccess;
 }

@@ -2,19 +2,21 @@
 // in shared memory.
 //
 // One lane runs one sample's Wilson LE_v run as Alg. 2 and Alg. 4 state it
-// (draw k at node u is the Philox draw (u, k, i, 0)); one more warp per CTA runs
-// the samples' absorbed walks (walk_tasks.cuh).  A run on a graph of a thousand
+// (draw k at node u is the Philox draw (u, k, i, 0)).  A run on a graph of a thousand
 // nodes is a chain of a few thousand dependent steps that more walkers do not
 // shorten (its walks hit the root late and meet each other before), so what
 // counts is the time of one step: about 300 cycles here, where the 1-byte
 // kernel waits for three L2 or DRAM accesses per step.
 //
 // State per sample: one tree bit, one path bit and one byte of draws per node,
-// laid out word by word across the warp's lanes (word w of lane l at w * 32 + l),
-// so lanes at different nodes never share a bank.  The current loop-erased path
-// is a stack of 16-bit node ids in the workspace, its two topmost entries in
-// registers (most loops have two nodes).  From its 255th draw on a node is
-// counted in a 32-bit word of the workspace.
+// laid out word by word across the warp's samples (word w of lane l at w * lanes +
+// l).  The current loop-erased path is a stack of 16-bit node ids in the workspace,
+// its two topmost entries in registers (most loops have two nodes).  From its 255th
+// draw on a node is counted in a 32-bit word of the workspace.
+//
+// Lanes of a warp in different phases of a step wait for each other, so a warp has
+// few samples: 10000 samples of an Erdos-Renyi graph of 1000 nodes take 5.1 / 4.3 /
+// 4.3 / 4.3 ms with 22 / 8 / 4 / 2 per warp (the 1-byte kernel: 9.4 ms).
 #include "walk_tasks.cuh"
 
 namespace {
@@ -26,10 +28,10 @@ enum : uint32_t { S_CLAIM = 0, S_SCAN, S_STEP, S_ADD };
 
 // LOCAL: packed arcs and row records are in shared memory.
 template <bool CV, bool LOCAL>
-__global__ void __launch_bounds__(288) lewalk_small_kernel(LapSampleLaunch p, LapBlockLaunch b, uint32_t lanes)
+__global__ void __launch_bounds__(512) lewalk_small_kernel(LapSampleLaunch p, LapBlockLaunch b, uint32_t lanes)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warps = (blockDim.x >> 5) - 1u;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const uint32_t n = (uint32_t)p.g.n, v = (uint32_t)p.root;
     const Graph<true> g{p.g.rowinfo, p.g.col, b.arcs, b.bw, b.bo, policy_evict_last()};
     unsigned long long *const arcs = reinterpret_cast<unsigned long long *>(smem);
@@ -41,19 +43,14 @@ __global__ void __launch_bounds__(288) lewalk_small_kernel(LapSampleLaunch p, La
             rows[x] = make_uint2((uint32_t)p.g.rowinfo[x].x, (uint32_t)p.g.rowinfo[x].y);
         __syncthreads();
     }
-    if (warp == warps) {
-        walk_tasks<CV, true>(p, b, g);
-        return;
-    }
     const uint32_t nw = (n + 31u) >> 5, nk = (n + 3u) >> 2;
-    uint32_t *const tree = state0 + warp * (2u * nw + nk) * 32u + lane, *const path = tree + nw * 32u;
-    uint8_t *const draws = reinterpret_cast<uint8_t *>(path + nw * 32u);
-    const uint64_t slot = (blockIdx.x * (uint64_t)warps + warp) * 32ull + lane;
+    uint32_t *const tree = state0 + warp * (2u * nw + nk) * lanes + lane, *const path = tree + nw * lanes;
+    uint8_t *const draws = reinterpret_cast<uint8_t *>(path + nw * lanes);
+    const uint64_t slot = (blockIdx.x * (uint64_t)warps + warp) * lanes + lane;
     uint16_t *const stk = reinterpret_cast<uint16_t *>(b.stacks) + slot * b.stack_entries;
     uint32_t *const many = b.sweep + slot * n;
     const uint32_t key0 = (uint32_t)p.seed, key1 = (uint32_t)(p.seed >> 32);
-    auto bit = [](const uint32_t *a, uint32_t u) { return (a[(u >> 5) * 32u] >> (u & 31u)) & 1u; };
-    auto draws_at = [&](uint32_t u) -> uint8_t & { return draws[(u >> 2) * 128u + (u & 3u)]; };
+    auto draws_at = [&](uint32_t u) -> uint8_t & { return draws[(u >> 2) * (4u * lanes) + (u & 3u)]; };
     auto row = [&](uint32_t u, uint32_t &off, uint32_t &deg) {
         if (LOCAL) {
             const uint2 r = rows[u];
@@ -73,7 +70,7 @@ __global__ void __launch_bounds__(288) lewalk_small_kernel(LapSampleLaunch p, La
     while (phase != 0xFFu) {
         if (phase == S_STEP) {
             // u has just been reached.
-            const uint32_t m = 1u << (u & 31u), x = (u >> 5) * 32u;
+            const uint32_t m = 1u << (u & 31u), x = (u >> 5) * lanes;
             if (tree[x] & m) {
                 add = sp;
                 phase = S_ADD;
@@ -82,13 +79,13 @@ __global__ void __launch_bounds__(288) lewalk_small_kernel(LapSampleLaunch p, La
                 if (on & m) {
                     // A loop closed at u: its nodes leave the path.
                     if (below == u && sp > 1u) {
-                        path[(top >> 5) * 32u] &= ~(1u << (top & 31u));
+                        path[(top >> 5) * lanes] &= ~(1u << (top & 31u));
                         path[x] &= ~m;
                         sp -= 2u;
                     } else {
                         for (;;) {
                             const uint32_t w = stk[--sp];
-                            path[(w >> 5) * 32u] &= ~(1u << (w & 31u));
+                            path[(w >> 5) * lanes] &= ~(1u << (w & 31u));
                             if (w == u) break;
                         }
                     }
@@ -127,7 +124,7 @@ __global__ void __launch_bounds__(288) lewalk_small_kernel(LapSampleLaunch p, La
         if (phase == S_ADD) {
             // The path joins the tree: a few nodes at a time, or all its bits.
             if (add > 24u) {
-                for (uint32_t x = 0; x < nw * 32u; x += 32u) {
+                for (uint32_t x = 0; x < nw * lanes; x += lanes) {
                     tree[x] |= path[x];
                     path[x] = 0u;
                 }
@@ -137,8 +134,8 @@ __global__ void __launch_bounds__(288) lewalk_small_kernel(LapSampleLaunch p, La
                 for (int t = 0; t < 4 && add > 0u; ++t) {
                     if (add != sp) w = stk[add - 1u];
                     --add;
-                    tree[(w >> 5) * 32u] |= 1u << (w & 31u);
-                    path[(w >> 5) * 32u] &= ~(1u << (w & 31u));
+                    tree[(w >> 5) * lanes] |= 1u << (w & 31u);
+                    path[(w >> 5) * lanes] &= ~(1u << (w & 31u));
                 }
             }
             if (add == 0u) phase = S_SCAN;
@@ -146,8 +143,8 @@ __global__ void __launch_bounds__(288) lewalk_small_kernel(LapSampleLaunch p, La
         if (phase == S_SCAN) {
             // The next start: the first node not in the tree.
             sp = 0;
-            uint32_t t = ~tree[s * 32u];
-            if (t == 0u && ++s < nw) t = ~tree[s * 32u];
+            uint32_t t = ~tree[s * lanes];
+            if (t == 0u && ++s < nw) t = ~tree[s * lanes];
             if (t) {
                 u = s * 32u + (uint32_t)__ffs(t) - 1u;
                 row(u, off, deg);
@@ -162,9 +159,9 @@ __global__ void __launch_bounds__(288) lewalk_small_kernel(LapSampleLaunch p, La
             q = atomicAdd(&p.acc->claim, 1u);
             if (q >= p.count) break;
             i = p.first + q;
-            for (uint32_t x = 0; x < (2u * nw + nk) * 32u; x += 32u) tree[x] = 0u;
-            if (n & 31u) tree[(nw - 1u) * 32u] = ~((1u << (n & 31u)) - 1u);
-            tree[(v >> 5) * 32u] |= 1u << (v & 31u);
+            for (uint32_t x = 0; x < (2u * nw + nk) * lanes; x += lanes) tree[x] = 0u;
+            if (n & 31u) tree[(nw - 1u) * lanes] = ~((1u << (n & 31u)) - 1u);
+            tree[(v >> 5) * lanes] |= 1u << (v & 31u);
             s = 0;
             sp = 0;
             top = 0;
@@ -177,6 +174,7 @@ __global__ void __launch_bounds__(288) lewalk_small_kernel(LapSampleLaunch p, La
 }
 
 constexpr uint64_t kSmem = 227ull << 10;
+constexpr uint64_t kLanes = 4;         // samples per warp, where 16 warps hold the call's
 
 }  // namespace
 
@@ -184,38 +182,42 @@ bool lap_small_plan(int32_t n, int64_t arcs, uint64_t count, uint64_t slots_opt,
                     LapSmallPlan *out)
 {
     LapSmallPlan pl;
-    const uint64_t nn = (uint64_t)n, per_warp = 128ull * (2ull * ((nn + 31ull) / 32ull) + (nn + 3ull) / 4ull);
+    const uint64_t nn = (uint64_t)n, per_lane = 4ull * (2ull * ((nn + 31ull) / 32ull) + (nn + 3ull) / 4ull);
     const uint64_t graph = 8ull * (uint64_t)arcs + 8ull * nn;
     if (num_sms < 1) num_sms = 1;
-    if (per_warp > kSmem || nn > 65535ull) return false;
+    if (per_lane > kSmem || nn > 65535ull) return false;
     uint64_t want = count;
     if (slots_opt && slots_opt < want) want = slots_opt;
     if (want == 0) want = 1;
-    const uint64_t per_sm = (want + num_sms - 1) / num_sms;
-    uint64_t warps = (per_sm + 31ull) / 32ull;
-    if (warps > 8) warps = 8;
-    // The graph's copy stays if it leaves room for the warps the call can use.
-    pl.local = graph + per_warp <= kSmem && (kSmem - graph) / per_warp >= (warps < 3 ? warps : 3);
-    const uint64_t fit = (kSmem - (pl.local ? graph : 0ull)) / per_warp;
-    if (warps > fit) warps = fit;
-    uint64_t lanes = (per_sm + warps - 1) / warps;
-    if (lanes > 32) lanes = 32;
+    uint64_t per_sm = (want + num_sms - 1) / num_sms;
+    if (per_sm > 16ull * 32ull) per_sm = 16ull * 32ull;
+    // The graph's copy stays if it leaves room for the samples the call can use,
+    // or for 96.
+    pl.local = graph < kSmem && (kSmem - graph) / per_lane >= (per_sm < 96ull ? per_sm : 96ull);
+    const uint64_t fit = (kSmem - (pl.local ? graph : 0ull)) / per_lane;
+    if (per_sm > fit) per_sm = fit;
+    // Few samples per warp: lanes in different phases of a step wait for each other.
+    uint64_t warps = (per_sm + kLanes - 1ull) / kLanes;
+    if (warps > 16) warps = 16;
+    const uint64_t lanes = (per_sm + warps - 1) / warps;
+    if (warps * lanes > fit) warps = fit / lanes;
     const uint64_t blocks = (want + warps * lanes - 1) / (warps * lanes);
     pl.warps = (int)warps;
+    pl.walk_ctas = 4ull * num_sms;
     pl.lanes = (uint32_t)lanes;
     pl.blocks = blocks < (uint64_t)num_sms ? blocks : (uint64_t)num_sms;
-    pl.smem = (pl.local ? graph : 0ull) + warps * per_warp;
+    pl.smem = (pl.local ? graph : 0ull) + warps * lanes * per_lane;
     // Workspace: path words of the loop-included paths, the stacks, the words of
     // nodes drawn often.
     const uint64_t entries = (nn + 7ull) & ~7ull;
-    const uint64_t slots = pl.blocks * warps * 32ull;
+    const uint64_t slots = pl.blocks * warps * lanes;
     const uint64_t stacks = (2ull * entries + 4ull * nn) * slots + 512ull;
     const uint64_t path_bytes = paths ? 8ull * nn : 0ull;
     if (stacks + path_bytes > ws_bytes) return false;
     pl.b.path_lanes = 0;
     if (paths) {
         pl.b.path_lanes = (ws_bytes - stacks) / path_bytes;
-        if (pl.b.path_lanes > pl.blocks * 32ull) pl.b.path_lanes = pl.blocks * 32ull;
+        if (pl.b.path_lanes > pl.walk_ctas * 32ull) pl.b.path_lanes = pl.walk_ctas * 32ull;
     }
     pl.words_bytes = pl.b.path_lanes * path_bytes;
     pl.stack_offset = (pl.words_bytes + 255ull) & ~255ull;
@@ -236,6 +238,6 @@ cudaError_t lap_launch_sample_small(const LapSampleLaunch &p, const LapSmallPlan
     if (e != cudaSuccess) return e;
     uint32_t lanes = pl.lanes;
     void *args[3] = {const_cast<LapSampleLaunch *>(&p), const_cast<LapBlockLaunch *>(&pl.b), &lanes};
-    e = cudaLaunchKernel(kernel, dim3((unsigned)pl.blocks), dim3((unsigned)(32 * (pl.warps + 1))), args, (size_t)pl.smem, st);
+    e = cudaLaunchKernel(kernel, dim3((unsigned)pl.blocks), dim3((unsigned)(32 * pl.warps)), args, (size_t)pl.smem, st);
     return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -14,8 +14,9 @@ from paper_2311_10290_gb300.lap import LAP_OPT_KERNEL, LAP_OPT_SLOTS, LapGraph  
 
 @pytest.mark.parametrize("maker,splits,root", [(lambda: I.path(2), [5], 0), (lambda: I.ba(33, 2, seed=1), [64], -1),
                                                (lambda: I.ba(4097, 3, seed=2), [1, 200], -1),
-                                               (lambda: I.rmat(14, 8, seed=3), [100], 77), (lambda: I.path(300), [20], 299)],
-                         ids=["two_nodes", "n33", "n4097", "rmat", "path"])
+                                               (lambda: I.rmat(14, 8, seed=3), [100], 77), (lambda: I.path(300), [20], 299),
+                                               (lambda: I.er(12000, 6 / 12000, seed=4), [150], -1)],
+                         ids=["two_nodes", "n33", "n4097", "rmat", "path", "parts"])
 def test_trees_equal_wide_kernel(maker, splits, root):
     g = maker()
     out = []
