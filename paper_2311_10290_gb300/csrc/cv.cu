@@ -13,6 +13,7 @@
 #include "lap_internal.h"
 #include "philox.cuh"
 #include "rows.cuh"
+#include "walk_tasks.cuh"
 
 namespace {
 
@@ -101,29 +102,53 @@ struct IntNeighbourSum {
     __device__ void end(int32_t u, int2, T t) const { S[u] = t; }
 };
 
-// One thread per (node, repetition): a walk from u absorbed at v; step t uses
-// Philox counter (t, u, rep, 3).
-__global__ void hitting_walks_kernel(LapDevGraph g, int32_t v, uint64_t seed, uint32_t reps, uint64_t limit,
-                                     unsigned long long *__restrict__ sums, unsigned int *status)
+// v-absorbed walks from every node, `reps` each.  A lane that has finished a walk
+// takes its next one at once, so a warp never waits for its longest walk, and the
+// step's draw is computed while the column load is in flight.  Bound by the
+// longest walk of the call, one L2 access per step with packed arcs (30,000 nodes,
+// 16 walks each: 5.3 -> 4.5 ms against a warp per 32 walks at a time and two
+// dependent accesses per step).
+template <bool PACK>
+__global__ void __launch_bounds__(128) hitting_walks_kernel(LapDevGraph dg, const unsigned long long *__restrict__ arcs, uint32_t bw,
+                                                            uint32_t bo, int32_t v, uint64_t seed, uint32_t reps,
+                                                            uint64_t limit, unsigned long long *__restrict__ sums,
+                                                            unsigned int *status)
 {
-    const uint64_t total = (uint64_t)g.n * reps;
+    const lap_walks::Graph<PACK> g{dg.rowinfo, dg.col, arcs, bw, bo, lap_walks::policy_evict_last()};
+    const uint64_t total = (uint64_t)dg.n * reps, lanes = (uint64_t)gridDim.x * blockDim.x;
     const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-    for (uint64_t pair = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; pair < total;
-         pair += (uint64_t)gridDim.x * blockDim.x) {
-        const int32_t u = (int32_t)(pair / reps);
-        const uint32_t rep = (uint32_t)(pair % reps);
-        uint64_t t = 0;
-        int32_t x = u;
-        bool bad = false;
-        while (x != v) {
-            ++t;
-            if (t > limit) { bad = true; break; }
-            const int2 r = g.rowinfo[x];
-            x = g.col[r.x + (int64_t)lap::below(lap::philox_r64((uint32_t)t, (uint32_t)u, rep, 3u, k0, k1), (uint64_t)r.y)];
+    uint64_t pair = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, t = 0, r = 0;
+    uint32_t u = 0, x = (uint32_t)v, rep = 0, off = 0, deg = 1;
+    bool active = false, bad = false;
+    for (;;) {
+        if (!active) {
+            if (pair >= total) break;
+            u = (uint32_t)(pair / reps);
+            rep = (uint32_t)(pair % reps);
+            pair += lanes;
+            if (u == (uint32_t)v) continue;
+            g.row(u, off, deg);
+            r = lap::philox_r64(1u, u, rep, 3u, k0, k1);
+            t = 0;
+            active = true;
         }
-        if (bad) atomicOr(status, (unsigned int)LAP_DEV_STEP_LIMIT);
-        else if (t) atomicAdd(&sums[u], (unsigned long long)t);
+        ++t;
+        if (t > limit) {
+            bad = true;
+            active = false;
+            continue;
+        }
+        const uint64_t a = g.arc(off + lap_walks::below32(r, deg));
+        r = lap::philox_r64((uint32_t)(t + 1u), u, rep, 3u, k0, k1);
+        x = g.target(a);
+        if (x == (uint32_t)v) {
+            atomicAdd(&sums[u], (unsigned long long)t);
+            active = false;
+        } else {
+            g.next_row(a, x, off, deg);
+        }
     }
+    if (bad) atomicOr(status, (unsigned int)LAP_DEV_STEP_LIMIT);
 }
 
 __device__ double block_sum(double x)
@@ -437,14 +462,22 @@ cudaError_t lap_launch_potential(const int2 *rowinfo, const int32_t *col, int32_
     return lap_rows::launch_rows(IntNeighbourSum{h, S}, rowinfo, col, n, hubs, st);
 }
 
-cudaError_t lap_launch_hitting_walks(const LapDevGraph &g, int32_t root, uint64_t seed, uint32_t reps, uint64_t limit,
-                                     unsigned long long *sums, unsigned int *status, int num_sms, cudaStream_t st)
+cudaError_t lap_launch_hitting_walks(const LapDevGraph &g, const unsigned long long *arcs, int32_t root, uint64_t seed,
+                                     uint32_t reps, uint64_t limit, unsigned long long *sums, unsigned int *status,
+                                     int num_sms, cudaStream_t st)
 {
     const uint64_t total = (uint64_t)g.n * reps;
     uint64_t grid = (total + 127) / 128;
     const uint64_t cap = (uint64_t)(num_sms > 0 ? num_sms : 1) * 16;
     if (grid > cap) grid = cap;
-    hitting_walks_kernel<<<(unsigned)(grid < 1 ? 1 : grid), 128, 0, st>>>(g, root, seed, reps, limit, sums, status);
+    if (grid < 1) grid = 1;
+    uint32_t bw = 1, bo = 1;
+    if (arcs) {
+        lap_pack_bits(g.n, g.arcs, &bw, &bo);
+        hitting_walks_kernel<true><<<(unsigned)grid, 128, 0, st>>>(g, arcs, bw, bo, root, seed, reps, limit, sums, status);
+    } else {
+        hitting_walks_kernel<false><<<(unsigned)grid, 128, 0, st>>>(g, arcs, bw, bo, root, seed, reps, limit, sums, status);
+    }
     return cudaGetLastError();
 }
 

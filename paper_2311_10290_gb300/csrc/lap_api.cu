@@ -1222,7 +1222,7 @@ lap_status lap_hitting_walks(lap_graph *g, uint32_t reps, uint64_t seed, uint64_
     unsigned int *status = reinterpret_cast<unsigned int *>(g->d_red);
     LAP_CUDA(g, cudaMemsetAsync(status, 0, sizeof(unsigned int), g->stream));
     const uint64_t limit = g->step_limit ? g->step_limit : default_step_limit(g->n);
-    LAP_CUDA(g, lap_launch_hitting_walks(LapDevGraph{g->d_rowinfo, g->d_col, g->n, g->arcs}, g->root, seed, reps, limit,
+    LAP_CUDA(g, lap_launch_hitting_walks(LapDevGraph{g->d_rowinfo, g->d_col, g->n, g->arcs}, g->d_arcs, g->root, seed, reps, limit,
                                          reinterpret_cast<unsigned long long *>(sums_dev), status, g->num_sms,
                                          g->stream));
     unsigned int h = 0;

@@ -313,8 +313,9 @@ cudaError_t lap_launch_features(const int2 *rowinfo, const int32_t *col, const i
                                 double *scratch, float *feat, cudaStream_t st);
 cudaError_t lap_launch_potential(const int2 *rowinfo, const int32_t *col, int32_t n, LapHubs hubs, const double *phi, long long *h,
                                  long long *S, cudaStream_t st);
-cudaError_t lap_launch_hitting_walks(const LapDevGraph &g, int32_t root, uint64_t seed, uint32_t reps, uint64_t limit,
-                                     unsigned long long *sums, unsigned int *status, int num_sms, cudaStream_t st);
+cudaError_t lap_launch_hitting_walks(const LapDevGraph &g, const unsigned long long *arcs, int32_t root, uint64_t seed,
+                                     uint32_t reps, uint64_t limit, unsigned long long *sums, unsigned int *status,
+                                     int num_sms, cudaStream_t st);   // arcs: packed arcs or NULL
 cudaError_t lap_launch_cv_finalize(const int2 *rowinfo, int32_t n, int32_t root, uint64_t omega,
                                    const unsigned long long *rep1, const unsigned long long *cnt2,
                                    const long long *a1, const long long *S1, double beta1,
