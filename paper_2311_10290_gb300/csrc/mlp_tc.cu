@@ -6,9 +6,11 @@
 // BF16 where they enter a product, biases, accumulators, bias gradients and
 // the loss in FP32.
 //
-// One CTA of 128 threads works on tiles of 128 rows: row r of a tile is TMEM
-// lane r and thread r (warp w reads lanes 32w..32w+31).  Per tile, one thread
-// issues each layer's products (M = 128, N = 16..64, K in steps of 16) and
+// 128 threads work on a tile of 128 rows: row r of a tile is TMEM lane r and
+// thread r (warp w reads lanes 32w..32w+31).  Training has one such group per CTA;
+// the forward pass four, each with its own operand buffers, TMEM columns and
+// mbarrier, so that eight tiles per SM hide each other's waits.  Per tile, one
+// thread issues each layer's products (M = 128, N = 16..64, K in steps of 16) and
 // commits them to an mbarrier; all threads wait on it, read their row's
 // accumulators with tcgen05.ld, apply bias and ReLU, and write the next
 // operand to shared memory.  Training adds the backward pass:
@@ -83,7 +85,6 @@ struct Small {
 };
 
 constexpr uint32_t align_up(uint32_t x, uint32_t a) { return (x + a - 1) / a * a; }
-constexpr uint32_t kFwdBytes = align_up(kFwdOps, 16) + (uint32_t)sizeof(Small);
 constexpr uint32_t kTrainBytes = align_up(kTrainF, 16) + (uint32_t)sizeof(Small);
 
 // Instruction descriptor, kind::f16: FP32 accumulator (bits 4-5 = 1), BF16 A
@@ -201,17 +202,193 @@ __device__ __forceinline__ float warp_sum(float x)
     return x;
 }
 
-// Forward (TRAIN = false: Y = MLP(X)) or loss and gradient (TRAIN = true:
-// G and loss accumulate the batch's MSE gradient and loss).
-template <bool TRAIN>
-__global__ void __launch_bounds__(kThreads, TRAIN ? 1 : 4)
-    mlp_tc_kernel(const float *__restrict__ P, const float *__restrict__ X, const float *__restrict__ T, int64_t n,
-                  float wk0, float wk1, float inv_n, float *__restrict__ Y, float *__restrict__ G,
-                  float *__restrict__ loss)
+// ------------------------------------------------------------ forward
+
+// Bound by instruction issue (about 400 per warp and tile, of which 64 x 2 biases and
+// the conversions are most) once a tile's three round trips to the tensor core are
+// hidden.  One group per CTA, four CTAs per SM, rows loaded when their tile began
+// and 64 accumulators held per thread: 45 us on 1,000,003 rows; now 35 us.
+constexpr int kGroups = 4;
+constexpr uint32_t fSW1 = 0;                            // B  [64 x 16]   W1
+constexpr uint32_t fSW2 = fSW1 + 64 * 16 * 2;           // B  [64 x 64]   W2
+constexpr uint32_t fSW3 = fSW2 + 64 * 64 * 2;           // B  [16 x 64]   W3 (rows 0..1)
+constexpr uint32_t fX = fSW3 + 16 * 64 * 2;             // A  [128 x 16]  X (features 0..7), per group
+constexpr uint32_t kXBytes = kTile * 16 * 2;
+constexpr uint32_t fH = fX + kGroups * kXBytes;         // A  [128 x 64]  H1, then H2, per group
+constexpr uint32_t kHBytes = kTile * 64 * 2;
+constexpr uint32_t kForwardOps = fH + kGroups * kHBytes;
+
+struct ForwardSmall {
+    unsigned long long bar[kGroups];
+    uint32_t tmem;
+    uint32_t fail[kGroups];          // a wait of the group has run out
+    float b3[kOut];
+    alignas(16) float b1[kHid];
+    alignas(16) float b2[kHid];
+};
+constexpr uint32_t kForwardBytes = align_up(kForwardOps, 16) + (uint32_t)sizeof(ForwardSmall);
+
+// 32 consecutive FP32 columns of this thread's lane.
+__device__ __forceinline__ void tm_ld32(uint32_t taddr, float *v)
+{
+    uint32_t r[32];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n\t"
+                 "tcgen05.wait::ld.sync.aligned;"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                 : "r"(taddr)
+                 : "memory");
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// relu of two values, as BF16 (rounded first: the same value; a NaN gives 0).
+__device__ __forceinline__ uint32_t relu2(float lo, float hi)
+{
+    __nv_bfloat162 v = __hmax2(__floats2bfloat162_rn(lo, hi), __floats2bfloat162_rn(0.f, 0.f));
+    return *reinterpret_cast<uint32_t *>(&v);
+}
+
+// H = relu(Z + b) of this thread's row, from TMEM to the next layer's A operand.
+__device__ __forceinline__ void hidden_row(uint32_t taddr, const float *b, unsigned char *sm, uint32_t base, int r)
+{
+#pragma unroll
+    for (int c = 0; c < 64; c += 32) {
+        float z[32];
+        tm_ld32(taddr + c, z);
+#pragma unroll
+        for (int g = 0; g < 32; g += 8) {
+            const float4 p = *reinterpret_cast<const float4 *>(b + c + g), q = *reinterpret_cast<const float4 *>(b + c + g + 4);
+            *reinterpret_cast<uint4 *>(sm + base + cm_off(r, c + g, 64)) =
+                make_uint4(relu2(z[g] + p.x, z[g + 1] + p.y), relu2(z[g + 2] + p.z, z[g + 3] + p.w),
+                           relu2(z[g + 4] + q.x, z[g + 5] + q.y), relu2(z[g + 6] + q.z, z[g + 7] + q.w));
+        }
+    }
+}
+
+// Y = MLP(X).  Tile t of group g of CTA b: t = (turn * kGroups + g) * CTAs + b, so
+// few rows spread over all CTAs first.
+__global__ void __launch_bounds__(kThreads * kGroups, 2)
+    mlp_tc_forward_kernel(const float *__restrict__ P, const float *__restrict__ X, int64_t n, float *__restrict__ Y)
 {
     extern __shared__ __align__(1024) unsigned char sm[];
-    constexpr uint32_t kOps = TRAIN ? align_up(kTrainF, 16) : align_up(kFwdOps, 16);
-    constexpr uint32_t kCols = TRAIN ? 256u : 128u;
+    ForwardSmall &s = *reinterpret_cast<ForwardSmall *>(sm + align_up(kForwardOps, 16));
+    const int tid = threadIdx.x, warp = tid >> 5, group = tid / kThreads, r = tid % kThreads;
+    const uint32_t s0 = smem_u32(sm), bar = smem_u32(&s.bar[group]);
+    volatile uint32_t *const fail = &s.fail[group];
+    const int64_t step = (int64_t)gridDim.x * kGroups * kTile;
+    int64_t row = ((int64_t)group * gridDim.x + blockIdx.x) * kTile + r;
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 xa = zero4, xb = zero4;                         // the row of the tile to come
+    if (row < n) {
+        xa = *reinterpret_cast<const float4 *>(X + row * kIn);
+        xb = *reinterpret_cast<const float4 *>(X + row * kIn + 4);
+    }
+    // Weights; zeros in the unused columns and rows.
+    for (uint32_t i = tid; i < fH / 16; i += kThreads * kGroups) reinterpret_cast<uint4 *>(sm)[i] = make_uint4(0, 0, 0, 0);
+    float w2[kHid * kHid / (kThreads * kGroups)];
+#pragma unroll
+    for (int k = 0; k < kHid * kHid / (kThreads * kGroups); ++k) w2[k] = P[oW2 + k * kThreads * kGroups + tid];
+    const float w1 = P[oW1 + tid], w3 = tid < kOut * kHid ? P[oW3 + tid] : 0.f;
+    static_assert(kHid * kIn == kThreads * kGroups, "one W1 entry per thread");
+    if (tid < kHid) {
+        s.b1[tid] = P[ob1 + tid];
+        s.b2[tid] = P[ob2 + tid];
+    }
+    if (tid < kOut) s.b3[tid] = P[ob3 + tid];
+    __syncthreads();
+    st_bf16(sm, fSW1 + cm_off(tid / kIn, tid % kIn, 16), w1);
+#pragma unroll
+    for (int k = 0; k < kHid * kHid / (kThreads * kGroups); ++k) {
+        const int i = k * kThreads * kGroups + tid;
+        st_bf16(sm, fSW2 + cm_off(i / kHid, i % kHid, 64), w2[k]);
+    }
+    if (tid < kOut * kHid) st_bf16(sm, fSW3 + cm_off(tid / kHid, tid % kHid, 64), w3);
+    if (r == 0) {
+        *fail = 0u;
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(bar) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(&s.tmem)),
+                     "r"(64u * kGroups) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    fence_proxy();
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tm = s.tmem + 64u * group;                              // the group's columns
+    const uint32_t lane_tm = tm + ((uint32_t)((warp & 3) * 32) << 16);     // this warp's 32 lanes
+    const uint32_t x_op = fX + kXBytes * group, h_op = fH + kHBytes * group;
+    uint32_t parity = 0;
+
+    auto group_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(kThreads) : "memory"); };
+    // Operands written by the group's threads, then one layer's products.
+    auto layer = [&](uint32_t a, uint32_t b, int K, int steps, uint32_t id) {
+        fence_proxy();
+        fence_before();
+        group_sync();
+        if (r == 0 && !*fail) {
+            fence_after();
+            gemm(tm, s0 + a, s0 + b, K, steps, id, false);
+            commit(bar);
+        }
+        // (After a wait that ran out, no product is issued and no wait begun.)
+        if (!*fail && !wait_phase(bar, parity)) *fail = 1u;
+        parity ^= 1u;
+        fence_after();
+    };
+
+    for (int64_t first = row - r; first < n; first += step, row += step) {
+        *reinterpret_cast<uint4 *>(sm + x_op + cm_off(r, 0, 16)) =
+            make_uint4(pack2(xa.x, xa.y), pack2(xa.z, xa.w), pack2(xb.x, xb.y), pack2(xb.z, xb.w));
+        xa = xb = zero4;
+        if (row + step < n) {
+            xa = *reinterpret_cast<const float4 *>(X + (row + step) * kIn);
+            xb = *reinterpret_cast<const float4 *>(X + (row + step) * kIn + 4);
+        }
+        layer(x_op, fSW1, 16, 1, idesc(128, 64));
+        hidden_row(lane_tm, s.b1, sm, h_op, r);
+        layer(h_op, fSW2, 64, 4, idesc(128, 64));
+        hidden_row(lane_tm, s.b2, sm, h_op, r);
+        layer(h_op, fSW3, 64, 4, idesc(128, 16));
+        float y[16];
+        tm_ld16(lane_tm, y);
+        if (row < n) *reinterpret_cast<float2 *>(Y + row * kOut) = make_float2(y[0] + s.b3[0], y[1] + s.b3[1]);
+    }
+
+    group_sync();
+    if (*fail) {
+        // A product did not complete in time: wait once more (bounded) for the
+        // one in flight, then report through the outputs.
+        wait_phase(bar, 0u);
+        wait_phase(bar, 1u);
+        const float nan = __int_as_float(0x7fc00000);
+        for (int64_t q = ((int64_t)group * gridDim.x + blockIdx.x) * kTile + r; q < n; q += step)
+            *reinterpret_cast<float2 *>(Y + q * kOut) = make_float2(nan, nan);
+    }
+    fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(s.tmem), "r"(64u * kGroups) : "memory");
+    }
+}
+
+// ------------------------------------------------------------ training
+
+// Loss and gradient: G and loss accumulate the batch's MSE gradient and loss.
+__global__ void __launch_bounds__(kThreads, 1)
+    mlp_tc_train_kernel(const float *__restrict__ P, const float *__restrict__ X, const float *__restrict__ T, int64_t n,
+                        float wk0, float wk1, float inv_n, float *__restrict__ G, float *__restrict__ loss)
+{
+    extern __shared__ __align__(1024) unsigned char sm[];
+    constexpr uint32_t kOps = align_up(kTrainF, 16);
+    constexpr uint32_t kCols = 256u;
     Small &s = *reinterpret_cast<Small *>(sm + kOps);
     float *sF = reinterpret_cast<float *>(sm + oF);
     const int tid = threadIdx.x, warp = tid >> 5;
@@ -223,12 +400,12 @@ __global__ void __launch_bounds__(kThreads, TRAIN ? 1 : 4)
     for (int i = tid; i < kHid * kHid; i += kThreads) {
         const int u = i / kHid, j = i % kHid;
         st_bf16(sm, oSW2 + cm_off(u, j, 64), P[oW2 + i]);
-        if (TRAIN) st_bf16(sm, oSW2T + cm_off(j, u, 64), P[oW2 + i]);
+        st_bf16(sm, oSW2T + cm_off(j, u, 64), P[oW2 + i]);
     }
     for (int i = tid; i < kOut * kHid; i += kThreads) {
         const int o = i / kHid, j = i % kHid;
         st_bf16(sm, oSW3 + cm_off(o, j, 64), P[oW3 + i]);
-        if (TRAIN) st_bf16(sm, oSW3T + cm_off(j, o, 16), P[oW3 + i]);
+        st_bf16(sm, oSW3T + cm_off(j, o, 16), P[oW3 + i]);
     }
     if (tid < kHid) {
         s.b1[tid] = P[ob1 + tid];
@@ -271,10 +448,8 @@ __global__ void __launch_bounds__(kThreads, TRAIN ? 1 : 4)
             x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
             *reinterpret_cast<uint4 *>(sm + oX + cm_off(tid, 0, 16)) =
                 make_uint4(pack2(x[0], x[1]), pack2(x[2], x[3]), pack2(x[4], x[5]), pack2(x[6], x[7]));
-            if (TRAIN) {
 #pragma unroll
-                for (int f = 0; f < kIn; ++f) st_bf16(sm, oB2 + cm_off(f, tid, 128), x[f]);
-            }
+            for (int f = 0; f < kIn; ++f) st_bf16(sm, oB2 + cm_off(f, tid, 128), x[f]);
         }
         fence_proxy();
         fence_before();
@@ -300,10 +475,8 @@ __global__ void __launch_bounds__(kThreads, TRAIN ? 1 : 4)
             h[j] = fmaxf(z, 0.f);
         }
         st_row64(sm, oH1, tid, h);
-        if (TRAIN) {
 #pragma unroll
-            for (int j = 0; j < kHid; ++j) st_bf16(sm, oB1 + cm_off(j, tid, 128), h[j]);
-        }
+        for (int j = 0; j < kHid; ++j) st_bf16(sm, oB1 + cm_off(j, tid, 128), h[j]);
         fence_proxy();
         fence_before();
         __syncthreads();
@@ -326,10 +499,8 @@ __global__ void __launch_bounds__(kThreads, TRAIN ? 1 : 4)
             h[j] = fmaxf(z, 0.f);
         }
         st_row64(sm, oH2, tid, h);
-        if (TRAIN) {
 #pragma unroll
-            for (int j = 0; j < kHid; ++j) st_bf16(sm, oT + cm_off(128 + j, tid, 128), h[j]);
-        }
+        for (int j = 0; j < kHid; ++j) st_bf16(sm, oT + cm_off(128 + j, tid, 128), h[j]);
         fence_proxy();
         fence_before();
         __syncthreads();
@@ -348,11 +519,6 @@ __global__ void __launch_bounds__(kThreads, TRAIN ? 1 : 4)
         tm_ld16(lane_tm + 0, y);
         y[0] += s.b3[0];
         y[1] += s.b3[1];
-        if (!TRAIN) {
-            if (valid) *reinterpret_cast<float2 *>(Y + row * kOut) = make_float2(y[0], y[1]);
-            fence_before();    // this tile's TMEM reads precede the next tile's products
-            continue;
-        }
 
         // ---- loss and dY = 2 w_k (y - t) / N (rows beyond n contribute nothing)
         float dy0 = 0.f, dy1 = 0.f, l = 0.f;
@@ -455,18 +621,8 @@ __global__ void __launch_bounds__(kThreads, TRAIN ? 1 : 4)
         // A product did not complete in time: wait once more (bounded) for the
         // phase in flight, then report through the outputs.
         wait_phase(bar, parity ^ 1u);
-        if (TRAIN) {
-            if (tid == 0) atomicAdd(loss, __int_as_float(0x7fc00000));
-        } else {
-            for (int64_t tile = blockIdx.x; tile * kTile < n; tile += gridDim.x) {
-                const int64_t row = tile * kTile + tid;
-                if (row < n) {
-                    const float nan = __int_as_float(0x7fc00000);
-                    *reinterpret_cast<float2 *>(Y + row * kOut) = make_float2(nan, nan);
-                }
-            }
-        }
-    } else if (TRAIN && any) {
+        if (tid == 0) atomicAdd(loss, __int_as_float(0x7fc00000));
+    } else if (any) {
         const int m = warp * 32 + (tid & 31);     // TMEM lane = row of the gradient products
         float v[kHid];
         if (warp < 2) {
@@ -510,18 +666,18 @@ cudaError_t lap_launch_mlp_tc(const float *P, const float *X, const float *T, in
     if (T) {
         // One CTA per SM (shared memory), 256 TMEM columns each.
         const int grid = (int)(tiles < sms ? tiles : sms);
-        cudaError_t e = cudaFuncSetAttribute(mlp_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(mlp_tc_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)kTrainBytes);
         if (e != cudaSuccess) return e;
-        mlp_tc_kernel<true><<<grid, kThreads, kTrainBytes, st>>>(P, X, T, n, wk0, wk1, 1.f / (float)n, Y, G, loss);
+        mlp_tc_train_kernel<<<grid, kThreads, kTrainBytes, st>>>(P, X, T, n, wk0, wk1, 1.f / (float)n, G, loss);
     } else {
-        // Up to four CTAs per SM: 4 x 128 TMEM columns fill the SM's 512.
-        const int64_t cap = (int64_t)sms * 4;
+        // Two CTAs per SM: 2 x 256 TMEM columns fill the SM's 512.
+        const int64_t cap = (int64_t)sms * 2;
         const int grid = (int)(tiles < cap ? tiles : cap);
-        cudaError_t e = cudaFuncSetAttribute(mlp_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kFwdBytes);
+        cudaError_t e = cudaFuncSetAttribute(mlp_tc_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)kForwardBytes);
         if (e != cudaSuccess) return e;
-        mlp_tc_kernel<false><<<grid, kThreads, kFwdBytes, st>>>(P, X, nullptr, n, 0.f, 0.f, 0.f, Y, nullptr, nullptr);
+        mlp_tc_forward_kernel<<<grid, kThreads * kGroups, kForwardBytes, st>>>(P, X, n, Y);
     }
     return cudaGetLastError();
 }
