@@ -1469,8 +1469,7 @@ lap_status lap_mlp_loss_grad(const float *params_dev, const float *x_dev, const 
     if (!params_dev || !x_dev || !t_dev || !grad_dev || !loss_dev || rows <= 0)
         return fail(nullptr, LAP_ERR_INVALID_ARG, "bad MLP arguments");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
-    cudaError_t e = cudaMemsetAsync(grad_dev, 0, sizeof(float) * LAP_MLP_PARAMS, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(loss_dev, 0, sizeof(float), st);
+    cudaError_t e = lap_launch_mlp_clear(grad_dev, loss_dev, st);
     if (e == cudaSuccess) e = launch_mlp(params_dev, x_dev, t_dev, rows, w0, w1, nullptr, grad_dev, loss_dev, st);
     return e == cudaSuccess ? LAP_OK : cuda_fail(nullptr, e, "lap_mlp_loss_grad");
 }

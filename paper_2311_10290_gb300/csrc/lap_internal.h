@@ -335,6 +335,7 @@ cudaError_t lap_launch_beta2_reduce(const unsigned long long *y1, const unsigned
                                     int64_t count, double *red, double *out, cudaStream_t st);
 // MLP forward (T = nullptr) or loss and gradient: mlp_tc.cu (tcgen05, TMEM
 // accumulators) or mlp.cu (mma.sync), per lap_mlp_select.
+cudaError_t lap_launch_mlp_clear(float *G, float *loss, cudaStream_t st);   // zeroes gradient and loss
 cudaError_t lap_launch_mlp_tc(const float *P, const float *X, const float *T, int64_t n, float wk0, float wk1,
                               float *Y, float *G, float *loss, cudaStream_t st);
 cudaError_t lap_launch_mlp_mma_sync(const float *P, const float *X, const float *T, int64_t n, float wk0,

