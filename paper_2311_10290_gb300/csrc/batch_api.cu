@@ -1,6 +1,16 @@
 // Host side of include/lap_batch.h: packed arenas of many graphs, the work
-// queue, CUDA-graph capture of one run (resets, persistent sampler, finalize),
-// re-runs of withdrawn samples, and the autotuner.
+// queue, CUDA-graph capture of one run (resets, sampling, finalize), re-runs of
+// withdrawn samples, and the autotuner.
+//
+// A run with the default launch options samples every graph with the kernels
+// of single graphs (sampler_cta.cu), side by side on parallel branches of the
+// captured graph, each with a share of the workspace.  The persistent sampler
+// (sampler_batch.cu, a lane per sample across all graphs) runs where LANES,
+// CLAIM, BLOCK or STACK are set, where the workspace does not hold the branches,
+// and, beside the branches, for graphs that the kernels of single graphs do not hold
+// or whose long first walks fill its lanes (plan_branches).  24 graphs of 1,000 to 100,000 nodes, 512
+// samples each: 565 ms persistent, 215 ms on branches, bound by the longest walks
+// of one Erdos-Renyi graph.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -27,6 +37,8 @@ struct lap_batch {
 
     int32_t *d_col = nullptr;
     int2 *d_rowinfo = nullptr;
+    unsigned long long *d_arcs = nullptr;            // packed arcs (lap_launch_pack_arcs) of the graphs with packed[g]
+    std::vector<char> packed;
     unsigned long long *d_rep1 = nullptr, *d_cnt2 = nullptr, *d_scratch = nullptr;
     double *d_ldiag = nullptr, *d_ecc = nullptr, *d_red = nullptr;
     LapBatchGraph *d_graphs = nullptr;
@@ -51,16 +63,21 @@ struct lap_batch {
 
     cudaStream_t stream = nullptr;
     cudaStream_t cap_stream = nullptr;
-    cudaStream_t rerun_streams[8] = {};
-    cudaEvent_t rerun_done[8] = {};
+    cudaStream_t branch_streams[20] = {};            // branches of a captured run; re-runs
+    cudaEvent_t branch_done[20] = {};
+    std::vector<int32_t> root_degree, max_degree;
+    cudaEvent_t fork = nullptr;
     cudaGraphExec_t exec = nullptr;
     bool key_valid = false;
     uint64_t key_samples = 0, key_seed = 0, key_lanes = 0;
     uint32_t key_claim = 0, key_stack = 0, key_paths = 0;
     int key_order = -1, key_block = -1;
+    bool key_cta = false;                // the captured run may take the branches ...
+    bool exec_cta = false;               // ... and does
     int64_t captures = 0;
 
     uint64_t lanes_opt = 0;
+    bool tuned = false;                  // lanes and claim come from the autotuner
     uint32_t claim_opt = 1;
     int order_opt = 0;
     int block_opt = 0;
@@ -71,6 +88,7 @@ struct lap_batch {
     uint64_t seed = 0;
     bool ran = false;
     bool checked = false;
+    bool ran_cta = false;                // the last run's samples were run on branches
     int64_t reruns = 0;
 
     lap_status sticky = LAP_OK;
@@ -80,7 +98,9 @@ struct lap_batch {
 namespace {
 
 thread_local std::string g_batch_error = "no error";
-constexpr int kRerunStreams = 8;
+constexpr int kBranches = 16, kWalkBranches = 4;
+constexpr int kRerunStreams = 8;                     // of the branch streams
+constexpr uint64_t kPackBytes = 96ull << 20;         // packed arcs that stay in L2
 
 lap_status bfail(lap_batch *b, lap_status s, const std::string &msg)
 {
@@ -111,12 +131,14 @@ void free_batch(lap_batch *b)
 {
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
-    for (int k = 0; k < 8; ++k) {
-        if (b->rerun_streams[k]) cudaStreamDestroy(b->rerun_streams[k]);
-        if (b->rerun_done[k]) cudaEventDestroy(b->rerun_done[k]);
+    for (int k = 0; k < kBranches + kWalkBranches; ++k) {
+        if (b->branch_streams[k]) cudaStreamDestroy(b->branch_streams[k]);
+        if (b->branch_done[k]) cudaEventDestroy(b->branch_done[k]);
     }
+    if (b->fork) cudaEventDestroy(b->fork);
     cudaFree(b->d_col);
     cudaFree(b->d_rowinfo);
+    cudaFree(b->d_arcs);
     cudaFree(b->d_rep1);
     cudaFree(b->d_cnt2);
     cudaFree(b->d_scratch);
@@ -233,14 +255,20 @@ lap_status ensure_workspace(lap_batch *b)
     return LAP_OK;
 }
 
-// Descriptors with this run's sample count, and the unit queue.
-lap_status upload_plan(lap_batch *b, uint64_t samples, uint32_t claim)
+// Descriptors with this run's sample count, and the unit queue (led by the units
+// of the graphs in `first`).
+lap_status upload_plan(lap_batch *b, uint64_t samples, uint32_t claim, const std::vector<int32_t> *first = nullptr)
 {
     for (auto &d : b->h_graphs) d.count = (uint32_t)samples;
     B_CUDA(b, cudaMemcpyAsync(b->d_graphs, b->h_graphs.data(), sizeof(LapBatchGraph) * b->h_graphs.size(),
                               cudaMemcpyHostToDevice, b->stream));
     std::vector<uint2> units;
     build_units(b->G, b->n.data(), b->order_opt, samples, claim, units);
+    if (first && !first->empty()) {
+        std::vector<char> lead((size_t)b->G, 0);
+        for (int32_t g : *first) lead[(size_t)g] = 1;
+        std::stable_partition(units.begin(), units.end(), [&](const uint2 &u) { return lead[u.x] != 0; });
+    }
     if (units.size() > b->units_cap) {
         cudaFree(b->d_units);
         b->d_units = nullptr;
@@ -285,7 +313,179 @@ LapBatchLaunch make_launch(const lap_batch *b, uint64_t seed, uint64_t lanes, ui
     return p;
 }
 
-// Captures one run: counter resets, the sampler, the finalize of every graph.
+lap_status ensure_branches(lap_batch *b)
+{
+    if (!b->fork) B_CUDA(b, cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming));
+    for (int k = 0; k < kBranches + kWalkBranches; ++k) {
+        if (!b->branch_streams[k]) B_CUDA(b, cudaStreamCreateWithFlags(&b->branch_streams[k], cudaStreamNonBlocking));
+        if (!b->branch_done[k]) B_CUDA(b, cudaEventCreateWithFlags(&b->branch_done[k], cudaEventDisableTiming));
+    }
+    return LAP_OK;
+}
+
+// The graphs' launches on branches: graphs in claim order, each to the branch
+// with the fewest nodes so far.  A branch's share of the workspace is what its
+// largest plan asks for, scaled down where all together ask for more than there is.
+// Fewer branches where a graph's plan does not fit its share; false if it does not
+// fit the whole workspace.
+struct Branches {
+    int count = 0;
+    std::vector<int32_t> rest;           // graphs left to the persistent sampler
+    std::vector<uint64_t> offset;        // of a branch's share of the workspace (and its end)
+    std::vector<int32_t> order;
+    std::vector<int> branch;             // of order[k]
+    std::vector<LapCtaPlan> plan;        // of order[k]
+};
+bool plan_branches(const lap_batch *b, uint64_t samples, Branches *out)
+{
+    if (samples >= (1ull << 30)) return false;               // the kernels' sample tags
+    Branches br;
+    std::vector<uint2> units;
+    build_units(b->G, b->n.data(), b->order_opt, 1, 1, units);
+    LapCtaPlan pl;
+    auto plan = [&](int32_t graph, uint64_t bytes) {
+        const size_t g = (size_t)graph;
+        return lap_cta_plan(b->n[g], b->arcs[g], b->root_degree[g], b->max_degree[g], samples, 0, bytes, b->num_sms, false, false,
+                            b->packed[g] != 0, &pl);
+    };
+    // Graphs with long first walks (their plans have table_bytes) end sooner on
+    // branches while the persistent sampler would be waiting for their chains; with
+    // enough samples to fill its lanes it has the higher throughput (40,000 lanes:
+    // 9.4e9 walk steps/s, twice the branches' on such graphs).
+    std::vector<uint64_t> ask((size_t)b->G, 0);      // 0: no plan
+    std::vector<char> slow((size_t)b->G, 0);
+    uint64_t slow_samples = 0;
+    for (int32_t g = 0; g < b->G; ++g) {
+        if (!plan(g, 1ull << 50)) continue;
+        ask[(size_t)g] = pl.bytes() + 4096ull;
+        slow[(size_t)g] = !pl.small && pl.block.table_bytes > 0;
+        if (slow[(size_t)g]) slow_samples += samples;
+        if (!pl.small && pl.block.table_bytes > b->ws_bytes / 8ull) ask[(size_t)g] = 0;
+    }
+    const bool fill = slow_samples > 256ull * (uint64_t)b->num_sms;
+    std::vector<uint64_t> asks;
+    for (const uint2 &u : units) {
+        if (ask[u.x] == 0 || (fill && slow[u.x])) {
+            br.rest.push_back((int32_t)u.x);
+        } else {
+            br.order.push_back((int32_t)u.x);
+            asks.push_back(ask[u.x]);
+        }
+    }
+    const int32_t m = (int32_t)br.order.size();
+    // The persistent sampler's slots take the first half, if it has graphs.
+    const uint64_t base = br.rest.empty() ? 0ull : (b->ws_bytes / 2ull) & ~255ull;
+    if (m == 0 || (base && base < slot_bytes_of(b))) return false;
+    br.plan.resize((size_t)m);
+    for (br.count = std::min<int32_t>(kBranches, m); br.count >= 1; br.count /= 2) {
+        std::vector<uint64_t> load((size_t)br.count, 0), want((size_t)br.count, 0);
+        br.branch.clear();
+        for (int32_t k = 0; k < m; ++k) {
+            const size_t t = (size_t)(std::min_element(load.begin(), load.end()) - load.begin());
+            br.branch.push_back((int)t);
+            load[t] += (uint64_t)b->n[(size_t)br.order[(size_t)k]];
+            want[t] = std::max(want[t], asks[(size_t)k]);
+        }
+        double all = 0.0;
+        for (uint64_t w : want) all += (double)w;
+        const double have = (double)(b->ws_bytes - base), scale = all > have ? have / all : 1.0;
+        br.offset.assign(1, base);
+        for (uint64_t w : want) br.offset.push_back(br.offset.back() + ((uint64_t)((double)w * scale) & ~255ull));
+        bool ok = br.offset.back() <= b->ws_bytes;
+        for (int32_t k = 0; k < m && ok; ++k) {
+            const size_t t = (size_t)br.branch[(size_t)k];
+            ok = plan(br.order[(size_t)k], br.offset[t + 1] - br.offset[t]);
+            br.plan[(size_t)k] = pl;
+        }
+        if (!ok) continue;
+        *out = br;
+        return true;
+    }
+    return false;
+}
+
+// The globaltimer of the run's start, or of the end of a graph's last part.
+__global__ void stamp_kernel(unsigned long long *out)
+{
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    atomicMax(out, t);
+}
+
+// rest: the persistent sampler's launch, on the graphs of br.rest.
+cudaError_t launch_branches(lap_batch *b, Branches &br, const LapBatchLaunch &rest, uint64_t samples, uint64_t seed,
+                            cudaStream_t cs)
+{
+    stamp_kernel<<<1, 1, 0, cs>>>(&b->d_ctl->t0);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaEventRecord(b->fork, cs);
+    for (int t = 0; t < kBranches + kWalkBranches && e == cudaSuccess; ++t)
+        e = cudaStreamWaitEvent(b->branch_streams[t], b->fork, 0);
+    const int32_t m = (int32_t)br.order.size();
+    std::vector<LapSampleLaunch> launches((size_t)m);
+    for (int32_t k = 0; k < m; ++k) {
+        const int32_t g = br.order[(size_t)k];
+        const LapBatchGraph &d = b->h_graphs[(size_t)g];
+        char *ws = reinterpret_cast<char *>(b->ws) + br.offset[(size_t)br.branch[(size_t)k]];
+        LapSampleLaunch &p = launches[(size_t)k];
+        memset(&p, 0, sizeof(p));
+        p.g = LapDevGraph{d.rowinfo, d.col, d.n, d.arcs};
+        p.root = d.root;
+        p.seed = seed;
+        p.count = (uint32_t)samples;
+        p.rep1 = d.rep1;
+        p.cnt2 = d.cnt2;
+        p.acc = b->d_acc + g;
+        p.step_limit = d.step_limit;
+        p.num_sms = b->num_sms;
+        p.ustart_dev = &b->d_graphs[g].ustart;
+        p.ovf_ids = b->d_rerun_ids + (uint64_t)g * samples;
+        lap_cta_bind(p, br.plan[(size_t)k], ws, b->packed[(size_t)g] ? b->d_arcs + b->csr_arc_off[(size_t)g] : nullptr, 0);
+    }
+    // The absorbed walks, longest expected first (2m / d_v steps).
+    std::vector<int32_t> by_length((size_t)m);
+    std::iota(by_length.begin(), by_length.end(), 0);
+    auto length = [&](int32_t k) {
+        const size_t g = (size_t)br.order[(size_t)k];
+        return (double)b->arcs[g] / (double)b->root_degree[g];
+    };
+    std::stable_sort(by_length.begin(), by_length.end(), [&](int32_t x, int32_t y) { return length(x) > length(y); });
+    for (int32_t j = 0; j < m && e == cudaSuccess; ++j) {
+        const int32_t k = by_length[(size_t)j];
+        cudaStream_t st = b->branch_streams[kBranches + j % kWalkBranches];
+        e = lap_launch_cta_walks(launches[(size_t)k], br.plan[(size_t)k], st);
+        if (e != cudaSuccess) break;
+        stamp_kernel<<<1, 1, 0, st>>>(b->d_tdone + br.order[(size_t)k]);
+        e = cudaGetLastError();
+    }
+    for (int32_t k = 0; k < m && e == cudaSuccess; ++k) {
+        const LapCtaPlan &pl = br.plan[(size_t)k];
+        cudaStream_t st = b->branch_streams[br.branch[(size_t)k]];
+        // The branch's previous graph has left its own words there.
+        char *ws = reinterpret_cast<char *>(b->ws) + br.offset[(size_t)br.branch[(size_t)k]];
+        if (pl.words_bytes()) e = cudaMemsetAsync(ws, 0, pl.words_bytes(), st);
+        if (e == cudaSuccess) e = lap_launch_cta_wilson(launches[(size_t)k], pl, st);
+        if (e != cudaSuccess) break;
+        stamp_kernel<<<1, 1, 0, st>>>(b->d_tdone + br.order[(size_t)k]);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess && !br.rest.empty()) e = lap_launch_batch(rest, false, cs);
+    for (int t = 0; t < kBranches + kWalkBranches; ++t) {      // joined on errors too: the capture must end
+        const cudaError_t f = cudaEventRecord(b->branch_done[t], b->branch_streams[t]);
+        const cudaError_t h = cudaStreamWaitEvent(cs, b->branch_done[t], 0);
+        if (e == cudaSuccess) e = f != cudaSuccess ? f : h;
+    }
+    return e;
+}
+
+// Whether the launch options leave the choice of kernel open (loop-included
+// paths need words per node and lane, which the branches' shares do not hold).
+bool default_options(const lap_batch *b)
+{
+    return (b->tuned || (b->lanes_opt == 0 && b->claim_opt == 1)) && b->block_opt == 0 && b->stack_opt == 0 && b->paths_opt == 0;
+}
+
+// Captures one run: counter resets, the sampling, the finalize of every graph.
 lap_status capture(lap_batch *b, uint64_t samples, uint64_t seed, uint64_t lanes, uint32_t claim, int block)
 {
     if (b->exec) {
@@ -294,9 +494,20 @@ lap_status capture(lap_batch *b, uint64_t samples, uint64_t seed, uint64_t lanes
         b->exec = nullptr;
     }
     b->key_valid = false;
-    lap_status s = upload_plan(b, samples, claim);
+    Branches br;
+    const bool cta = default_options(b) && plan_branches(b, samples, &br);
+    lap_status s = upload_plan(b, samples, claim, cta ? &br.rest : nullptr);
     if (s != LAP_OK) return s;
-    const LapBatchLaunch p = make_launch(b, seed, lanes, claim, block);
+    if (cta && (s = ensure_branches(b)) != LAP_OK) return s;
+    LapBatchLaunch p = make_launch(b, seed, lanes, claim, block);
+    if (cta) {
+        // The graphs of br.rest alone: their units lead the queue, their slots are in
+        // the first half of the workspace.
+        const uint64_t own = (samples + claim - 1) / claim * br.rest.size(), fit = b->ws_bytes / 2ull / p.slot_bytes;
+        p.n_units = (uint32_t)own;
+        if (p.lanes > fit) p.lanes = fit;
+        if (p.lanes > samples * br.rest.size()) p.lanes = samples * br.rest.size();
+    }
     cudaStream_t cs = b->cap_stream;
     B_CUDA(b, cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     const size_t nb = sizeof(unsigned long long) * (size_t)b->total_n;
@@ -306,8 +517,8 @@ lap_status capture(lap_batch *b, uint64_t samples, uint64_t seed, uint64_t lanes
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_done, 0, sizeof(unsigned int) * (size_t)b->G, cs);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_tdone, 0, sizeof(unsigned long long) * (size_t)b->G, cs);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_ctl, 0, sizeof(LapBatchCtl), cs);
-    if (e == cudaSuccess) e = cudaMemsetAsync(&b->d_ctl->t0, 0xFF, sizeof(unsigned long long), cs);
-    if (e == cudaSuccess) e = lap_launch_batch(p, false, cs);
+    if (e == cudaSuccess && !cta) e = cudaMemsetAsync(&b->d_ctl->t0, 0xFF, sizeof(unsigned long long), cs);
+    if (e == cudaSuccess) e = cta ? launch_branches(b, br, p, samples, seed, cs) : lap_launch_batch(p, false, cs);
     if (e == cudaSuccess) e = lap_launch_finalize_batch(b->d_graphs, b->G, b->max_n, samples, b->d_red, cs);
     cudaGraph_t graph = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(cs, &graph);
@@ -319,6 +530,8 @@ lap_status capture(lap_batch *b, uint64_t samples, uint64_t seed, uint64_t lanes
         return bcuda(b, e, "capturing the batch run");
     }
     b->key_valid = true;
+    b->key_cta = default_options(b);
+    b->exec_cta = cta;
     b->key_samples = samples;
     b->key_seed = seed;
     b->key_lanes = lanes;
@@ -331,14 +544,11 @@ lap_status capture(lap_batch *b, uint64_t samples, uint64_t seed, uint64_t lanes
     return LAP_OK;
 }
 
-// Re-runs withdrawn samples with the 8-byte kernel, graph by graph, then
-// finalizes every graph again.
-lap_status rerun_withdrawn(lap_batch *b, uint32_t count)
+// Re-runs withdrawn samples {graph, id} with the 8-byte kernel, graph by graph,
+// then finalizes every graph again.
+lap_status rerun_withdrawn(lap_batch *b, std::vector<uint2> &ovf, uint32_t flags)
 {
-    if (count > b->ovf_cap) return bfail(b, LAP_ERR_CUDA, "internal error: overflow list exceeded");
-    std::vector<uint2> ovf(count);
-    B_CUDA(b, cudaMemcpyAsync(ovf.data(), b->d_ovf, sizeof(uint2) * count, cudaMemcpyDeviceToHost, b->stream));
-    B_CUDA(b, cudaStreamSynchronize(b->stream));
+    const uint32_t count = (uint32_t)ovf.size();
     std::stable_sort(ovf.begin(), ovf.end(), [](const uint2 &a, const uint2 &c) { return a.x < c.x; });
     std::vector<unsigned int> ids(count);
     for (uint32_t k = 0; k < count; ++k) ids[k] = ovf[k].y;
@@ -356,7 +566,7 @@ lap_status rerun_withdrawn(lap_batch *b, uint32_t count)
         B_CUDA(b, cudaEventRecord(ready, b->stream));
         for (size_t j = 0; j < group.size(); ++j) {
             const Job &jb = group[j];
-            cudaStream_t st = b->rerun_streams[j % kRerunStreams];
+            cudaStream_t st = b->branch_streams[j % kRerunStreams];
             B_CUDA(b, cudaStreamWaitEvent(st, ready, 0));
             const LapBatchGraph &d = b->h_graphs[jb.g];
             char *ws = reinterpret_cast<char *>(b->ws) + jb.ws_off;
@@ -381,22 +591,19 @@ lap_status rerun_withdrawn(lap_batch *b, uint32_t count)
             p.ids = b->d_rerun_ids + jb.a;
             p.paths = b->paths_opt;
             p.ustart = d.ustart;
+            p.flags = flags;
             B_CUDA(b, lap_launch_sample(p, st));
         }
         for (int k = 0; k < kRerunStreams && k < (int)group.size(); ++k) {
-            B_CUDA(b, cudaEventRecord(b->rerun_done[k], b->rerun_streams[k]));
-            B_CUDA(b, cudaStreamWaitEvent(b->stream, b->rerun_done[k], 0));
+            B_CUDA(b, cudaEventRecord(b->branch_done[k], b->branch_streams[k]));
+            B_CUDA(b, cudaStreamWaitEvent(b->stream, b->branch_done[k], 0));
         }
         group.clear();
         ws_used = meta_used = 0;
         return LAP_OK;
     };
-    if (!b->rerun_streams[0]) {
-        for (int k = 0; k < kRerunStreams; ++k) {
-            B_CUDA(b, cudaStreamCreateWithFlags(&b->rerun_streams[k], cudaStreamNonBlocking));
-            B_CUDA(b, cudaEventCreateWithFlags(&b->rerun_done[k], cudaEventDisableTiming));
-        }
-    }
+    lap_status bs = ensure_branches(b);
+    if (bs != LAP_OK) return bs;
     lap_status fs = LAP_OK;
     for (uint32_t a = 0; a < count && fs == LAP_OK;) {
         uint32_t c = a;
@@ -431,7 +638,7 @@ lap_status rerun_withdrawn(lap_batch *b, uint32_t count)
             b->sticky = LAP_ERR_STEP_LIMIT;
             return bfail(b, LAP_ERR_STEP_LIMIT, "graph " + std::to_string(g) + ": a re-run sample exceeded the step budget");
         }
-    b->reruns = count;
+    b->reruns += count;
     return LAP_OK;
 }
 
@@ -444,8 +651,17 @@ lap_status finish(lap_batch *b)
     if (!b->ran) return bfail(b, LAP_ERR_NO_SAMPLES, "lap_batch_run has not been called");
     if (b->checked) return LAP_OK;
     LapBatchCtl c;
+    std::vector<LapDevAcc> acc;
     B_CUDA(b, cudaMemcpyAsync(&c, b->d_ctl, sizeof(c), cudaMemcpyDeviceToHost, b->stream));
+    if (b->ran_cta) {
+        acc.resize((size_t)b->G);
+        B_CUDA(b, cudaMemcpyAsync(acc.data(), b->d_acc, sizeof(LapDevAcc) * acc.size(), cudaMemcpyDeviceToHost, b->stream));
+    }
     B_CUDA(b, cudaStreamSynchronize(b->stream));
+    for (const LapDevAcc &a : acc) {
+        c.status |= a.status;
+        if (a.ovf_count > b->omega) return bfail(b, LAP_ERR_CUDA, "internal error: overflow list exceeded");
+    }
     if (c.status & LAP_DEV_STEP_LIMIT) {
         b->sticky = LAP_ERR_STEP_LIMIT;
         b->meta_dirty = true;
@@ -457,10 +673,25 @@ lap_status finish(lap_batch *b)
         return bfail(b, LAP_ERR_CUDA, "internal error: sampler status " + std::to_string(c.status));
     }
     b->reruns = 0;
+    std::vector<uint2> ovf, wilson;
     if (c.ovf_count) {
-        s = rerun_withdrawn(b, c.ovf_count);
-        if (s != LAP_OK) return s;
+        if (c.ovf_count > b->ovf_cap) return bfail(b, LAP_ERR_CUDA, "internal error: overflow list exceeded");
+        ovf.resize(c.ovf_count);
+        B_CUDA(b, cudaMemcpyAsync(ovf.data(), b->d_ovf, sizeof(uint2) * ovf.size(), cudaMemcpyDeviceToHost, b->stream));
+        B_CUDA(b, cudaStreamSynchronize(b->stream));
     }
+    for (size_t g = 0; g < acc.size(); ++g) {
+        std::vector<unsigned int> ids(acc[g].ovf_count);
+        if (ids.empty()) continue;
+        B_CUDA(b, cudaMemcpyAsync(ids.data(), b->d_rerun_ids + (uint64_t)g * b->omega, sizeof(unsigned int) * ids.size(),
+                                  cudaMemcpyDeviceToHost, b->stream));
+        B_CUDA(b, cudaStreamSynchronize(b->stream));
+        for (unsigned int id : ids) wilson.push_back(make_uint2((unsigned int)g, id));
+    }
+    if (!ovf.empty() && (s = rerun_withdrawn(b, ovf, 0u)) != LAP_OK) return s;
+    // On branches, the absorbed walks do not depend on a sample's Wilson run: they
+    // stand when it is withdrawn.
+    if (!wilson.empty() && (s = rerun_withdrawn(b, wilson, LAP_SAMPLE_WILSON_ONLY)) != LAP_OK) return s;
     b->checked = true;
     return LAP_OK;
 }
@@ -599,6 +830,23 @@ lap_status lap_batch_create(int32_t n_graphs, const int32_t *n, const int32_t *c
     for (size_t g = 0; g < G && e == cudaSuccess; ++g)
         if (b->src[g] == (int32_t)g)
             e = lap_launch_rowinfo(d_row_ptr + b->csr_node_off[g] + (int64_t)g, n[g], b->d_rowinfo + b->csr_node_off[g], st);
+    // Packed arcs where a graph's stay in L2 (an allocation that fails leaves the
+    // plain columns).
+    b->packed.assign(G, 0);
+    bool any_packed = false;
+    for (size_t g = 0; g < G; ++g) {
+        b->packed[g] = n[g] <= (1 << 21) && 8ull * (uint64_t)b->arcs[g] <= kPackBytes;
+        any_packed = any_packed || b->packed[g];
+    }
+    if (e == cudaSuccess && any_packed && balloc(&b->d_arcs, (size_t)b->csr_arcs) != cudaSuccess) {
+        cudaGetLastError();
+        b->d_arcs = nullptr;
+        b->packed.assign(G, 0);
+    }
+    for (size_t g = 0; g < G && e == cudaSuccess; ++g)
+        if (b->packed[g] && b->src[g] == (int32_t)g)
+            e = lap_launch_pack_arcs(b->d_rowinfo + b->csr_node_off[g], b->d_col + b->csr_arc_off[g], n[g], b->arcs[g],
+                                     b->d_arcs + b->csr_arc_off[g], st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cudaFree(d_row_ptr);
     d_row_ptr = nullptr;
@@ -606,13 +854,17 @@ lap_status lap_batch_create(int32_t n_graphs, const int32_t *n, const int32_t *c
     // Roots: the highest degree, smallest id on ties, where none was given.
     e = cudaMemsetAsync(b->d_tdone, 0, sizeof(unsigned long long) * G, st);
     for (size_t g = 0; g < G && e == cudaSuccess; ++g)
-        if (b->roots[g] < 0) e = lap_launch_argmax_degree(b->d_rowinfo + b->csr_node_off[g], n[g], b->d_tdone + g, st);
+        e = lap_launch_argmax_degree(b->d_rowinfo + b->csr_node_off[g], n[g], b->d_tdone + g, st);
     std::vector<unsigned long long> best(G);
     if (e == cudaSuccess) e = cudaMemcpyAsync(best.data(), b->d_tdone, sizeof(unsigned long long) * G, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_bad(e, "root selection");
     for (size_t g = 0; g < G; ++g)
         if (b->roots[g] < 0) b->roots[g] = (int32_t)(0xFFFFFFFFu - (uint32_t)(best[g] & 0xFFFFFFFFull));
+    b->root_degree.resize(G);
+    b->max_degree.resize(G);
+    for (size_t g = 0; g < G; ++g) b->max_degree[g] = (int32_t)(best[g] >> 32);
+    for (size_t g = 0; g < G; ++g) b->root_degree[g] = row_ptr[g][b->roots[g] + 1] - row_ptr[g][b->roots[g]];
     // Connectivity: level-synchronous BFS of all graphs together (hop
     // distances kept in the ldiag arena, which holds 8 bytes per node).
     int32_t *hops = reinterpret_cast<int32_t *>(b->d_ldiag);
@@ -689,10 +941,12 @@ lap_status lap_batch_set_option(lap_batch *b, int32_t option, int64_t value)
     switch (option) {
     case LAP_BOPT_LANES:
         b->lanes_opt = (uint64_t)value;
+        b->tuned = false;
         return LAP_OK;
     case LAP_BOPT_CLAIM:
         if (value < 1 || value > 65536) return bfail(b, LAP_ERR_INVALID_ARG, "claim must be in [1, 65536]");
         b->claim_opt = (uint32_t)value;
+        b->tuned = false;
         return LAP_OK;
     case LAP_BOPT_ORDER:
         if (value > 2) return bfail(b, LAP_ERR_INVALID_ARG, "order must be 0, 1 or 2");
@@ -767,11 +1021,13 @@ lap_status lap_batch_run(lap_batch *b, uint64_t samples_per_graph, uint64_t seed
     const uint32_t claim = b->claim_opt;
     if (!b->key_valid || !b->exec || b->key_samples != samples_per_graph || b->key_seed != seed || b->key_lanes != lanes ||
         b->key_claim != claim || b->key_order != b->order_opt || b->key_block != block || b->key_stack != stack_cap_of(b) ||
-        b->key_paths != b->paths_opt) {
+        b->key_paths != b->paths_opt || b->key_cta != default_options(b)) {
         s = capture(b, samples_per_graph, seed, lanes, claim, block);
         if (s != LAP_OK) return s;
     }
     B_CUDA(b, cudaGraphLaunch(b->exec, b->stream));
+    b->ran_cta = b->exec_cta;
+    if (b->ran_cta) b->meta_dirty = true;            // the workspace holds other state than the slots'
     b->omega = samples_per_graph;
     b->seed = seed;
     b->ran = true;
@@ -862,6 +1118,7 @@ lap_status lap_batch_autotune(lap_batch *b, uint64_t samples_per_graph, uint64_t
     b->meta_dirty = false;
     b->lanes_opt = best_lanes;
     b->claim_opt = best_claim;
+    b->tuned = true;
     if (n_trials) *n_trials = rows;
     return LAP_OK;
 }

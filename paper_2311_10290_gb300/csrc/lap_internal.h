@@ -104,6 +104,7 @@ struct LapSampleLaunch {
     uint32_t flags;              // LAP_SAMPLE_* below
     uint32_t ustart;             // 0: the first absorbed walk (or path) starts at a uniform draw
                                  // (Alg. 2); s + 1: it starts at node s (single-source rows of L_v^{-1})
+    const uint32_t *ustart_dev;  // if set, the device word that walk_tasks reads instead of ustart
 };
 enum : uint32_t {
     LAP_SAMPLE_ONE_PER_LANE = 1u,   // wide kernel: lane j runs exactly sample first + j (j < count), so its
@@ -155,7 +156,8 @@ struct LapBlockPlan {
     uint64_t walk_ctas = 0;           // CTAs (of a warp) for the absorbed walks
     uint64_t slots = 0, smem = 0;     // CTAs (samples in flight), shared memory of each
     uint64_t words_bytes = 0;         // words and path words, zeroed when the layout grows
-    uint64_t path_offset = 0, stack_offset = 0, sweep_offset = 0, early_offset = 0;
+    uint64_t path_offset = 0, stack_offset = 0, sweep_offset = 0, early_offset = 0, bytes = 0;
+    uint64_t table_bytes = 0;         // the early tables of all samples of a call with long first walks
 };
 void lap_pack_bits(int32_t n, int64_t arcs, uint32_t *bw, uint32_t *bo);
 cudaError_t lap_launch_pack_arcs(const int2 *rowinfo, const int32_t *col, int32_t n, int64_t arcs,
@@ -171,7 +173,7 @@ struct LapSmallPlan {
     uint64_t walk_ctas = 0;           // CTAs (of a warp) for the absorbed walks
     uint32_t lanes = 0;               // lanes of a warp that take samples
     bool local = false;               // the graph is copied to shared memory
-    uint64_t slots = 0, blocks = 0, smem = 0, words_bytes = 0, stack_offset = 0, many_offset = 0;
+    uint64_t slots = 0, blocks = 0, smem = 0, words_bytes = 0, stack_offset = 0, many_offset = 0, bytes = 0;
 };
 bool lap_small_plan(int32_t n, int64_t arcs, uint64_t count, uint64_t slots_opt, uint64_t ws_bytes, int num_sms, bool paths,
                     LapSmallPlan *out);
@@ -183,6 +185,7 @@ struct LapCtaPlan {
     LapBlockPlan block;
     LapSmallPlan lane;
     uint64_t words_bytes() const { return small ? lane.words_bytes : block.words_bytes; }
+    uint64_t bytes() const { return small ? lane.bytes : block.bytes; }     // of workspace
 };
 bool lap_cta_plan(int32_t n, int64_t arcs, int32_t root_degree, int32_t max_degree, uint64_t count, uint64_t slots_opt, uint64_t ws_bytes, int num_sms, bool paths,
                   bool cv, bool pack, LapCtaPlan *out);

@@ -1114,8 +1114,10 @@ bool lap_block_plan(int32_t n, int64_t arcs, int32_t root_degree, int32_t max_de
     uint64_t m = ws_bytes > pl.early_offset + 64ull ? (ws_bytes - pl.early_offset - 64ull) / early_per : 0ull;
     if (m > count) m = count;
     b.early_count = (uint32_t)m;
+    pl.bytes = fixed_bytes + b.path_lanes * path_bytes + early_per * m + 64ull;
     // Where the first walk is long, a call whose tables do not fit runs in parts.
-    b.part = pass > 16ull * target && b.early_count > 0 && b.early_count < count ? b.early_count : (uint32_t)count;
+    if (pass > 16ull * target) pl.table_bytes = early_per * count;
+    b.part = pl.table_bytes && b.early_count > 0 && b.early_count < count ? b.early_count : (uint32_t)count;
     // Few samples per warp: a warp's lanes wait for each other.
     const uint64_t warps = 16ull * num_sms;
     const uint64_t l = (m + warps - 1) / warps;

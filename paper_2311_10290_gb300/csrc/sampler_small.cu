@@ -222,6 +222,7 @@ bool lap_small_plan(int32_t n, int64_t arcs, uint64_t count, uint64_t slots_opt,
     pl.words_bytes = pl.b.path_lanes * path_bytes;
     pl.stack_offset = (pl.words_bytes + 255ull) & ~255ull;
     pl.many_offset = pl.stack_offset + 2ull * entries * slots;
+    pl.bytes = pl.words_bytes + stacks;
     pl.b.stack_entries = entries;
     pl.slots = slots_opt && slots_opt < slots ? slots_opt : slots;
     *out = pl;

@@ -142,6 +142,7 @@ static __device__ void walk_tasks(const LapSampleLaunch &p, const LapBlockLaunch
     const uint32_t key0 = (uint32_t)p.seed, key1 = (uint32_t)(p.seed >> 32);
     const uint32_t v = (uint32_t)p.root;
     const uint64_t tasks = 2ull * p.count;
+    const uint32_t ustart = p.ustart_dev ? *p.ustart_dev : p.ustart;
     bool open = usable, active = false;
     uint32_t kind = 0, q = 0, u = v, off = 0, deg = 1, i = 0;
     uint64_t t = 0, r = 0;
@@ -168,8 +169,8 @@ static __device__ void walk_tasks(const LapSampleLaunch &p, const LapBlockLaunch
                     active = true;
                     tag = (unsigned long long)((b.tag_base + q + 1u) * 2u + kind) << 32;
                     if (kind == 0) {
-                        u = p.ustart ? p.ustart - 1u
-                                     : (uint32_t)lap::below(lap::philox_r64(0u, 0u, i, 1u, key0, key1), (uint64_t)p.g.n);
+                        u = ustart ? ustart - 1u
+                                   : (uint32_t)lap::below(lap::philox_r64(0u, 0u, i, 1u, key0, key1), (uint64_t)p.g.n);
                         g.row(u, off, deg);
                     } else {
                         const uint64_t a = g.arc((uint32_t)lap::below(lap::philox_r64(0u, 0u, i, 2u, key0, key1), (uint64_t)p.g.arcs));
