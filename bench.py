@@ -135,6 +135,21 @@ def parse():
 
 KERNEL_NAMES = {1: "lewalk_kernel (8-byte state)", 2: "lewalk_compact_kernel (1-byte state)",
                 3: "lewalk_group_kernel (several walkers per sample, 2-byte state)"}
+# Sampler kernels of a call: the 1-byte, 8-byte and several-walkers kernels run a
+# sample whole; the other two leave the absorbed walks to a kernel of their own,
+# and the block kernel its early phase.
+SAMPLER_LAUNCHES = {"lewalk_block_kernel": 3, "lewalk_small_kernel": 2}
+
+
+def kernel_label(stat, n, walkers=0):
+    """Name of the sampler that ran.  Kernel 3 with the automatic number of
+    walkers keeps the tree in shared memory where it fits; the benchmark's
+    graph of 1000 nodes (Erdos-Renyi) takes the small-graph kernel."""
+    if stat == 3 and walkers == 0 and n < 1_700_000:
+        if n <= 4096:
+            return "lewalk_small_kernel (state and graph in shared memory)"
+        return "lewalk_block_kernel (one CTA per sample, tree in shared memory)"
+    return KERNEL_NAMES[stat]
 
 
 def peaks():
@@ -1178,9 +1193,9 @@ def extra_workload(torch, LapGraph, name, args, params):
                               "wilson_steps_per_node_per_sample": wilson / B / g.n},
                "roofline": {"bound": "hbm", "achieved": alg / t_kernel / 1e9, "peak": peak, "unit": "GB/s",
                             "frac": alg / t_kernel / 1e9 / peak,
-                            "traffic": measured_traffic(KERNEL_NAMES[G.stat(LAP_STAT_LAST_KERNEL)], wilson),
+                            "traffic": measured_traffic(kernel_label(G.stat(LAP_STAT_LAST_KERNEL), g.n), wilson),
                             "traffic_note": "per launch, scaled from a small-case ncu capture by Wilson steps"},
-               "kernel": KERNEL_NAMES[G.stat(LAP_STAT_LAST_KERNEL)], "fallbacks": G.stat(LAP_STAT_FALLBACKS),
+               "kernel": kernel_label(G.stat(LAP_STAT_LAST_KERNEL), g.n), "fallbacks": G.stat(LAP_STAT_FALLBACKS),
                "kemeny_estimate": kc, "slots": G.slots, "generate_seconds": round(t_gen, 1)}
     finally:
         G.close()
@@ -1298,12 +1313,11 @@ def run_ours(args, rank, world):
     if args.ws_gb > 0:
         ws = min(ws, int(args.ws_gb * 1e9))
     G = LapGraph(g.row_ptr, g.col, workspace_bytes=ws)
-    from paper_2311_10290_gb300.lap import LAP_OPT_KERNEL, LAP_OPT_WALKERS, LAP_STAT_KERNEL
+    from paper_2311_10290_gb300.lap import LAP_OPT_KERNEL, LAP_OPT_WALKERS
     if args.kernel:
         G.set_option(LAP_OPT_KERNEL, args.kernel)
         G.set_option(LAP_OPT_WALKERS, args.walkers)
     v = G.set_root()
-    kernel_name = KERNEL_NAMES[G.stat(LAP_STAT_KERNEL)]
     B = args.batch
     total_steps = args.warmup + args.steps
     from paper_2311_10290_gb300.shard import allreduce_counts, id_range
@@ -1321,7 +1335,7 @@ def run_ours(args, rank, world):
         step()
     torch.cuda.synchronize()
     from paper_2311_10290_gb300.lap import LAP_STAT_LAST_KERNEL
-    kernel_name = KERNEL_NAMES[G.stat(LAP_STAT_LAST_KERNEL)]
+    kernel_name = kernel_label(G.stat(LAP_STAT_LAST_KERNEL), g.n, args.walkers if args.kernel else 0)
     c1a, c2a, sa = lap_counts(G.h, g.n)
     ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True),
            torch.cuda.Event(enable_timing=True)) for _ in range(args.steps)]
@@ -1397,7 +1411,7 @@ def run_ours(args, rank, world):
                      "traffic_note": "per launch, scaled from a small-case ncu capture by Wilson steps (profiles/)",
                      "kernel": kernel_name.split()[0], "kernel_ms": kernel_s * 1e3,
                      "peak_kind": peak_kind + " (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured" else peak_kind},
-        "gpu_launches": args.steps * 7,
+        "gpu_launches": args.steps * (6 + SAMPLER_LAUNCHES.get(kernel_name.split()[0], 1)),
     }
     if merged:
         res["merged_estimate"] = merged

@@ -71,14 +71,18 @@ typedef enum {
     LAP_OPT_STEP_LIMIT = 1,    /* per-sample budget on each of the three walks' steps; 0 = default
                                   (2^20 + 1024 n); the value is clamped to [1, 2^62] */
     LAP_OPT_SLOTS = 2,         /* samples kept in flight per launch; 0 = as many as the workspace holds */
-    LAP_OPT_BLOCK = 3,         /* threads per block of the sampler launch; 0 = automatic */
+    LAP_OPT_BLOCK = 3,         /* threads per block of the sampler launch (kernels 1 and 2, and kernel 3
+                                  with a number of walkers); 0 = automatic */
     LAP_OPT_CURSOR = 4,        /* first sample id of the next lap_sample (default 0); only before the
                                   first sample after lap_set_root.  Lets several processes or GPUs
                                   draw disjoint sample-id ranges whose counts add up exactly. */
-    LAP_OPT_KERNEL = 5,        /* 0 = automatic: kernel 3 for calls of at most 320 samples per SM
-                                  (1024 when the graph's arrays exceed 96 MB) on graphs of at
-                                  least 2^14 nodes when it applies, else kernel 2 when n < 2^27,
-                                  else kernel 1.
+    LAP_OPT_KERNEL = 5,        /* 0 = automatic: kernel 3 with the automatic number of walkers where
+                                  its state fits (a bit per node in an SM's shared memory, about
+                                  n < 1.7 million, and 20 n + 1.2 MB of workspace for one sample);
+                                  else kernel 3 with 8 or 16 walkers for calls of at most 320
+                                  samples per SM (1024 when the graph's arrays exceed 96 MB) on
+                                  graphs of at least 2^14 nodes, else kernel 2 when n < 2^27, else
+                                  kernel 1.
                                   1 = 8-byte state per node.
                                   2 = 1-byte state per node.  Kernel 2 keeps draw counts above 30
                                   (and, with LAP_OPT_PATHS = 1, path departure counts above 14) in
@@ -86,10 +90,16 @@ typedef enum {
                                   of two >= n, 256 to 8192.  A sample that does not fit kernel 2
                                   (more such nodes than the table holds, or a loop-erased path
                                   longer than the stack) is withdrawn and re-run with kernel 1.
-                                  3 = several walkers per sample (LAP_OPT_WALKERS lanes share one
-                                  Wilson run; 2 bytes of state per node): more independent memory
-                                  chains when a call has few samples, and each sample finishes
-                                  sooner.  Kernel 3 needs n < 2^22 and covers every estimator
+                                  3 = several walkers per sample.  With the automatic number of
+                                  walkers (LAP_OPT_WALKERS = 0) a CTA runs one sample with its tree
+                                  in shared memory, and graphs of up to 4096 nodes with long walks
+                                  to the root run a lane per sample with all state in shared
+                                  memory; the absorbed walks run beside the Wilson runs, on a
+                                  stream of the handle that is joined before the call's later
+                                  work.  A sample without progress for 4 s is withdrawn and re-run
+                                  with kernel 1.  Where that state does not fit, and with a
+                                  number of walkers, LAP_OPT_WALKERS lanes share one Wilson run
+                                  with 2 bytes of state per node.  That form needs n < 2^22 and covers every estimator
                                   form (LAP_OPT_PATHS 0 or 1, with or without the control
                                   variate; 2 more bytes per node with LAP_OPT_PATHS = 1).  Its
                                   samples that do not fit (a node drawn 1023 times, a path longer
@@ -108,9 +118,10 @@ typedef enum {
                                   expectations (so the same estimands), correlated with the Wilson
                                   counts, which lowers the variance of y1 - 2 y2 and of Y1 - Y2.
                                   Only before the first sample after lap_set_root. */
-    LAP_OPT_WALKERS = 9,       /* lanes per sample of kernel 3: 2, 4, 8 or 16; 0 (default) = 16 when
-                                  the call's samples times 16 lanes fit on the GPU at once (1280
-                                  lanes per SM), else 8.  The path stacks of a sample hold 8 x
+    LAP_OPT_WALKERS = 9,       /* lanes per sample of kernel 3: 2, 4, 8 or 16; 0 (default) =
+                                  automatic (see LAP_OPT_KERNEL; where the CTA form does not fit,
+                                  16 when the call's samples times 16 lanes fit on the GPU at
+                                  once, 1280 lanes per SM, else 8).  The path stacks of a sample hold 8 x
                                   LAP_OPT_STACK entries in all, shared out among its walkers;
                                   with 16 walkers a node drawn 511 times withdraws the sample.  They run the
                                   sample's Wilson run together (Section 3.4, stack representation:
@@ -131,9 +142,11 @@ typedef enum {
 
 /* Statistics for lap_get_stat. */
 typedef enum {
-    LAP_STAT_SLOTS = 1,        /* samples in flight per launch of a large call (LAP_STAT_KERNEL) with
+    LAP_STAT_SLOTS = 1,        /* samples in flight per launch with the layout of LAP_STAT_KERNEL and
                                   the current workspace (kernel 3: groups of walkers) */
-    LAP_STAT_KERNEL = 2,       /* kernel a large lap_sample call will use (1, 2 or 3) */
+    LAP_STAT_KERNEL = 2,       /* kernel (1, 2 or 3) whose slots LAP_STAT_SLOTS and lap_workspace_query
+                                  describe: the one a large call takes where kernel 3 with the
+                                  automatic number of walkers does not fit */
     LAP_STAT_FALLBACKS = 3,    /* samples re-run with kernel 1 after kernel 2 or 3 withdrew them, since
                                   lap_set_root (synchronises) */
     LAP_STAT_LAST_KERNEL = 4   /* kernel of the last lap_sample call (0 before any) */
@@ -176,8 +189,10 @@ lap_status lap_set_option(lap_graph *g, int32_t option, int64_t value);
  * sample in flight with kernel 1; with kernel 2, n rounded up to 256 (twice
  * that with LAP_OPT_PATHS = 1), plus 4 bytes per stack entry, plus the count
  * table (8 bytes times the next power of two >= n, 2 KB to 64 KB), rounded up
- * to 256).  lap_workspace_query returns the bytes the
- * current kernel needs to keep `slots` samples in flight.  lap_set_workspace lends the handle a caller-owned
+ * to 256; kernel 3 with the automatic number of walkers divides what there is,
+ * 20 bytes per node, path stacks of 1 to 4 MB and a table of its early phase per
+ * sample in flight).  lap_workspace_query returns the bytes the
+ * kernel of LAP_STAT_KERNEL needs to keep `slots` samples in flight.  lap_set_workspace lends the handle a caller-owned
  * device buffer (at least 8*n bytes, 256-byte aligned), which must stay alive
  * while the handle uses it; the handle zeroes it.  Without a workspace,
  * lap_sample allocates one itself (up to 1/2 of the free device memory).

@@ -30,9 +30,9 @@
 // apart (stride byte offset).
 //
 // Every wait on the mbarrier is bounded (1 s of %globaltimer); a wait that
-// runs out stops the CTA, waits once more (bounded) for its products in
-// flight, frees its TMEM and writes NaN to its outputs (forward) or to the
-// loss (training).
+// runs out stops the CTA (forward: the group), waits once more (bounded) for its
+// products in flight, frees its TMEM and writes NaN to its outputs (forward) or to
+// the loss (training).
 #include <cuda_bf16.h>
 
 #include "lap_internal.h"

@@ -1,6 +1,6 @@
-// Graph reads and the absorbed walks shared by the samplers that run a sample's
-// Wilson run and its absorbed walks in different warps (sampler_block.cu,
-// sampler_small.cu).
+// Graph reads shared by the samplers that leave the absorbed walks to a kernel of
+// their own (sampler_block.cu, sampler_small.cu), and these walks (launched by
+// sampler_cta.cu).
 #pragma once
 
 #include "lap_internal.h"
