@@ -1037,7 +1037,13 @@ bool lap_block_plan(int32_t n, int64_t arcs, int32_t root_degree, int32_t max_de
     b.idle_min = 12u;
     b.pair_min = 4u;
     b.unit_batch = nn > 200000 ? 4u : 2u;
-    b.cap_a = (uint32_t)(2ull * nn + 64ull < 8192ull ? 2ull * nn + 64ull : 8192ull);
+    // Paths of first walks have about sqrt(n) nodes, on sparse graphs a few times that;
+    // a sample whose path does not fit ends its early phase without a tree.  (With 4096
+    // entries at every size, 256 samples of Erdos-Renyi graphs of 10^6 nodes took over a
+    // minute; now 3.2 s, a lane per sample 11.9 s.)
+    uint64_t path = 4096ull;
+    while (path * path < 256ull * nn) path *= 2ull;
+    b.cap_a = (uint32_t)(2ull * nn + 64ull < 2ull * path ? 2ull * nn + 64ull : 2ull * path);
     b.cap_b = 512u;
     b.sweep_nodes = (uint32_t)(nn * 35ull / 100ull);
     b.sweep_rest = (uint32_t)(nn / 200ull < 64ull ? 64ull : nn / 200ull);
@@ -1072,7 +1078,7 @@ bool lap_block_plan(int32_t n, int64_t arcs, int32_t root_degree, int32_t max_de
     b.early_log2 = lg;
     b.early_entries = 1u << lg;
     b.early_nodes = (uint32_t)target;
-    b.early_cap = 4096u;
+    b.early_cap = (uint32_t)path;
     b.early_budget = 1u << 22;
     const uint64_t early_per = 4ull * b.early_entries + 4ull * b.early_cap + 4ull;
     // The workspace: at most half for the early tables (none if no sample fits

@@ -46,6 +46,7 @@ CASES = [("word_minus_1", lambda: I.ba(4127, 3, seed=1), 40, {}),
          ("star", lambda: I.star(5000), 64, dict(root=17)),
          ("grid", lambda: grid(66), 24, dict(root=0)),
          ("parts", lambda: I.er(12000, 6 / 12000, seed=9), 300, dict(ws=24 << 20, trace=True)),
+         ("long_paths", lambda: I.er(70000, 4 / 70000, seed=10), 8, {}),
          ("crossed_pairs", crossed_pairs, 200, dict(no_reruns=True))]
 
 
