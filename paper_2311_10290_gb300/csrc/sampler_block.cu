@@ -366,7 +366,12 @@ __global__ void __launch_bounds__(1024, 1) lewalk_block_kernel(LapSampleLaunch p
     unsigned long long acc1 = 0;
     unsigned int bad = 0;
 
-    auto group_sync = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(wilson) : "memory"); };
+    // All threads of the CTA, their warps converged first (the aligned barrier
+    // takes a warp as a whole).
+    auto group_sync = [&]() {
+        __syncwarp();
+        asm volatile("bar.sync 1, %0;" ::"r"(wilson) : "memory");
+    };
 
     for (;;) {
         // Claim a sample and clear the shared memory; the root and the
@@ -899,12 +904,16 @@ __global__ void __launch_bounds__(1024, 1) lewalk_block_kernel(LapSampleLaunch p
             pops = slow && !pops ? true : (slow && hard);
             first = false;
         }
+        // Read before the barrier: beyond it the first warps' walkers change both words,
+        // and a warp that saw them changed would leave with one barrier less than the
+        // others.
+        const bool complete = lds(ctl + cDone) >= n || lds(ctl + cStatus);
         if (j == 0) {
             sts(ctl + cIn, in);
             sts(ctl + cCursor, 0u);
         }
         group_sync();
-        if (lds(ctl + cDone) >= n || lds(ctl + cStatus)) break;
+        if (complete) break;
         }
         }
 
