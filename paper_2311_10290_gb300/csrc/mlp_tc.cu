@@ -339,6 +339,7 @@ __global__ void __launch_bounds__(kThreads * kGroups, 2)
         }
         // (After a wait that ran out, no product is issued and no wait begun.)
         if (!*fail && !wait_phase(bar, parity)) *fail = 1u;
+        __syncwarp();               // lanes leave the wait one by one; TMEM loads and barriers take whole warps
         parity ^= 1u;
         fence_after();
     };
