@@ -338,7 +338,7 @@ struct Branches {
 };
 bool plan_branches(const lap_batch *b, uint64_t samples, Branches *out)
 {
-    if (samples >= (1ull << 30)) return false;               // the kernels' sample tags
+    if (samples > LAP_TAGS) return false;
     Branches br;
     std::vector<uint2> units;
     build_units(b->G, b->n.data(), b->order_opt, 1, 1, units);

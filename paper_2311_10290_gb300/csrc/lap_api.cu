@@ -261,9 +261,9 @@ bool choose_cta(const lap_graph *g, uint64_t n_samples, LapCtaPlan *pl)
 lap_status launch_cta(lap_graph *g, LapSampleLaunch &p, LapCtaPlan &pl)
 {
     // The tagged words are zeroed when the workspace last held something else
-    // there, and when the tags (31 bits) run out.
+    // there, and when the tags run out.
     const uint64_t words = pl.words_bytes();
-    if (words > g->blk_clean || (uint64_t)g->tag_next + p.count + 1ull >= (1ull << 31)) {
+    if (words > g->blk_clean || (uint64_t)g->tag_next + p.count > LAP_TAGS) {
         LAP_CUDA(g, cudaMemsetAsync(g->ws, 0, words, g->stream));
         g->tag_next = 0;
     }

@@ -118,13 +118,21 @@ cudaError_t lap_launch_sample_compact(const LapSampleLaunch &p, cudaStream_t st)
 // p.stack_cap is the stack capacity of each walker
 cudaError_t lap_launch_sample_group(const LapSampleLaunch &p, int walkers, cudaStream_t st);
 
+// Tags of the workspace's words.  Sample s of the tag count (s < LAP_TAGS) marks
+// the words of its Wilson run and of its two absorbed walks apart: the border between
+// the two parts of the workspace moves with the samples in flight, so a call finds
+// words of either kind that earlier calls have left.  0 is nobody's tag.
+constexpr uint64_t LAP_TAGS = (1ull << 30) - 1ull;
+__host__ __device__ constexpr uint32_t lap_word_tag(uint32_t s) { return 4u * (s + 1u); }
+__host__ __device__ constexpr uint32_t lap_path_tag(uint32_t s, uint32_t kind) { return 4u * (s + 1u) + 2u + kind; }
+
 // sampler_block.cu: a CTA per sample, the tree bits in shared memory
 struct LapBlockLaunch {
     const unsigned long long *arcs;   // packed arcs (lap_launch_pack_arcs), or NULL
     uint32_t bw, bo;                  // their bits of target and row offset
     uint32_t fshift;                  // a filter bit covers 2^fshift nodes
     uint32_t lmask;                   // lock bit of node u: u & lmask
-    uint32_t tag_base;                // sample q of the launch has tag tag_base + q + 1
+    uint32_t tag_base;                // sample q of the launch has tag number tag_base + q
     unsigned long long *words;        // [slots * n] {tag 32 | k 32}
     unsigned long long *path_words;   // [path_lanes * n] departures of loop-included paths
     uint64_t path_lanes;

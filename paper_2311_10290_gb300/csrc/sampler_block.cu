@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(1024, 1) lewalk_block_kernel(LapSampleLaunch p
         const uint32_t q = lds(ctl + cClaim);
         if (q >= p.count) break;
         const uint32_t i = p.first + q;
-        d.tag = (unsigned long long)(b.tag_base + q + 1u) << 32;
+        d.tag = (unsigned long long)lap_word_tag(b.tag_base + q) << 32;
         const bool early = q < b.early_count;
         for (uint32_t x = j; x < nwords; x += wilson) {
             uint32_t t = x == v >> 5 ? 1u << (v & 31u) : 0u;

@@ -167,7 +167,7 @@ static __device__ void walk_tasks(const LapSampleLaunch &p, const LapBlockLaunch
                     t = 0;
                     m2 = 0.0;
                     active = true;
-                    tag = (unsigned long long)((b.tag_base + q + 1u) * 2u + kind) << 32;
+                    tag = (unsigned long long)lap_path_tag(b.tag_base + q, kind) << 32;
                     if (kind == 0) {
                         u = ustart ? ustart - 1u
                                    : (uint32_t)lap::below(lap::philox_r64(0u, 0u, i, 1u, key0, key1), (uint64_t)p.g.n);
