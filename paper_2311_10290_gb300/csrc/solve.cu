@@ -216,6 +216,7 @@ cudaError_t lap_run_lv_solve(const int2 *rowinfo, const int32_t *col, int32_t n,
         if (h.done || queued >= maxiter) break;
     }
     *iterations = h.it;
-    if (h.bb > 0.0) *residual = sqrt(h.rr) / sqrt(h.bb);
+    // (Not a number where b holds one: no tolerance is met by it.)
+    if (h.bb != 0.0) *residual = sqrt(h.rr) / sqrt(h.bb);
     return cudaSuccess;
 }
