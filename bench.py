@@ -133,23 +133,20 @@ def parse():
     return ap.parse_args()
 
 
+# Samplers by lap_form.
 KERNEL_NAMES = {1: "lewalk_kernel (8-byte state)", 2: "lewalk_compact_kernel (1-byte state)",
-                3: "lewalk_group_kernel (several walkers per sample, 2-byte state)"}
-# Sampler kernels of a call: the 1-byte, 8-byte and several-walkers kernels run a
-# sample whole; the other two leave the absorbed walks to a kernel of their own,
-# and the block kernel its early phase.
+                3: "lewalk_group_kernel (several walkers per sample, 2-byte state)",
+                4: "lewalk_block_kernel (one CTA per sample, tree in shared memory)",
+                5: "lewalk_small_kernel (state and graph in shared memory)"}
+# Launches of a call: the first three kernels run a sample whole; the other two leave the
+# absorbed walks to a kernel of their own, and the block kernel its early phase.
 SAMPLER_LAUNCHES = {"lewalk_block_kernel": 3, "lewalk_small_kernel": 2}
 
 
-def kernel_label(stat, n, walkers=0):
-    """Name of the sampler that ran.  Kernel 3 with the automatic number of
-    walkers keeps the tree in shared memory where it fits; the benchmark's
-    graph of 1000 nodes (Erdos-Renyi) takes the small-graph kernel."""
-    if stat == 3 and walkers == 0 and n < 1_700_000:
-        if n <= 4096:
-            return "lewalk_small_kernel (state and graph in shared memory)"
-        return "lewalk_block_kernel (one CTA per sample, tree in shared memory)"
-    return KERNEL_NAMES[stat]
+def kernel_label(G):
+    """Name of the sampler of the handle's last call."""
+    from paper_2311_10290_gb300.lap import LAP_STAT_LAST_FORM
+    return KERNEL_NAMES[G.stat(LAP_STAT_LAST_FORM)]
 
 
 def peaks():
@@ -1157,7 +1154,7 @@ def extra_workload(torch, LapGraph, name, args, params):
     """Plain throughput (1 warm-up and 1 timed launch of `extra_samples`
     samples) on another single-graph workload, then the control variate
     against plain on it when a trained network is given."""
-    from paper_2311_10290_gb300.lap import LAP_STAT_FALLBACKS, LAP_STAT_LAST_KERNEL, lap_counts
+    from paper_2311_10290_gb300.lap import LAP_STAT_FALLBACKS, lap_counts
     t0 = time.perf_counter()
     g = load_graph(name)
     t_gen = time.perf_counter() - t0
@@ -1193,9 +1190,9 @@ def extra_workload(torch, LapGraph, name, args, params):
                               "wilson_steps_per_node_per_sample": wilson / B / g.n},
                "roofline": {"bound": "hbm", "achieved": alg / t_kernel / 1e9, "peak": peak, "unit": "GB/s",
                             "frac": alg / t_kernel / 1e9 / peak,
-                            "traffic": measured_traffic(kernel_label(G.stat(LAP_STAT_LAST_KERNEL), g.n), wilson),
+                            "traffic": measured_traffic(kernel_label(G), wilson),
                             "traffic_note": "per launch, scaled from a small-case ncu capture by Wilson steps"},
-               "kernel": kernel_label(G.stat(LAP_STAT_LAST_KERNEL), g.n), "fallbacks": G.stat(LAP_STAT_FALLBACKS),
+               "kernel": kernel_label(G), "fallbacks": G.stat(LAP_STAT_FALLBACKS),
                "kemeny_estimate": kc, "slots": G.slots, "generate_seconds": round(t_gen, 1)}
     finally:
         G.close()
@@ -1334,8 +1331,7 @@ def run_ours(args, rank, world):
     for _ in range(args.warmup):
         step()
     torch.cuda.synchronize()
-    from paper_2311_10290_gb300.lap import LAP_STAT_LAST_KERNEL
-    kernel_name = kernel_label(G.stat(LAP_STAT_LAST_KERNEL), g.n, args.walkers if args.kernel else 0)
+    kernel_name = kernel_label(G)
     c1a, c2a, sa = lap_counts(G.h, g.n)
     ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True),
            torch.cuda.Event(enable_timing=True)) for _ in range(args.steps)]

@@ -149,8 +149,19 @@ typedef enum {
                                   automatic number of walkers does not fit */
     LAP_STAT_FALLBACKS = 3,    /* samples re-run with kernel 1 after kernel 2 or 3 withdrew them, since
                                   lap_set_root (synchronises) */
-    LAP_STAT_LAST_KERNEL = 4   /* kernel of the last lap_sample call (0 before any) */
+    LAP_STAT_LAST_KERNEL = 4,  /* kernel of the last lap_sample call (0 before any) */
+    LAP_STAT_LAST_FORM = 5,    /* lap_form of the last lap_sample call (0 before any) */
+    LAP_STAT_TREE_FORM = 6     /* lap_form that drew the last trees of the last lap_spantree_sample */
 } lap_stat;
+
+/* Samplers (kernel 3 is any of the last three). */
+typedef enum {
+    LAP_FORM_WIDE = 1,         /* kernel 1: a lane per sample, 8 bytes per node */
+    LAP_FORM_COMPACT = 2,      /* kernel 2: a lane per sample, 1 byte per node */
+    LAP_FORM_GROUP = 3,        /* kernel 3 with 2 to 16 lanes per sample */
+    LAP_FORM_BLOCK = 4,        /* kernel 3, a CTA per sample */
+    LAP_FORM_SMALL = 5         /* kernel 3, small graphs: a lane per sample, all state in shared memory */
+} lap_form;
 
 /* Library version as major*10000 + minor*100 + patch. */
 int32_t lap_version(void);

@@ -54,7 +54,9 @@ typedef enum {
     LAP_BSTAT_CLAIM = 2,         /* samples per work unit */
     LAP_BSTAT_UNITS = 3,         /* work units of the last run */
     LAP_BSTAT_RERUNS = 4,        /* samples of the last run re-run with the 8-byte kernel */
-    LAP_BSTAT_GRAPH_CAPTURES = 5 /* CUDA graphs captured by this handle so far */
+    LAP_BSTAT_GRAPH_CAPTURES = 5, /* CUDA graphs captured by this handle so far */
+    LAP_BSTAT_BRANCHES = 6       /* graphs of the last run that were sampled on branches (the others: by the
+                                    persistent sampler) */
 } lap_batch_stat_id;
 
 /*

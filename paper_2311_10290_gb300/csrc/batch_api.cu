@@ -73,7 +73,8 @@ struct lap_batch {
     uint32_t key_claim = 0, key_stack = 0, key_paths = 0;
     int key_order = -1, key_block = -1;
     bool key_cta = false;                // the captured run may take the branches ...
-    bool exec_cta = false;               // ... and does
+    bool exec_cta = false;               // ... and does ...
+    int32_t exec_branches = 0;           // ... for this many graphs
     int64_t captures = 0;
 
     uint64_t lanes_opt = 0;
@@ -88,7 +89,8 @@ struct lap_batch {
     uint64_t seed = 0;
     bool ran = false;
     bool checked = false;
-    bool ran_cta = false;                // the last run's samples were run on branches
+    bool ran_cta = false;                // the last run's samples were run on branches ...
+    int32_t ran_branches = 0;            // ... of this many graphs
     int64_t reruns = 0;
 
     lap_status sticky = LAP_OK;
@@ -532,6 +534,7 @@ lap_status capture(lap_batch *b, uint64_t samples, uint64_t seed, uint64_t lanes
     b->key_valid = true;
     b->key_cta = default_options(b);
     b->exec_cta = cta;
+    b->exec_branches = cta ? (int32_t)br.order.size() : 0;
     b->key_samples = samples;
     b->key_seed = seed;
     b->key_lanes = lanes;
@@ -1027,6 +1030,7 @@ lap_status lap_batch_run(lap_batch *b, uint64_t samples_per_graph, uint64_t seed
     }
     B_CUDA(b, cudaGraphLaunch(b->exec, b->stream));
     b->ran_cta = b->exec_cta;
+    b->ran_branches = b->exec_branches;
     if (b->ran_cta) b->meta_dirty = true;            // the workspace holds other state than the slots'
     b->omega = samples_per_graph;
     b->seed = seed;
@@ -1261,6 +1265,7 @@ lap_status lap_batch_stat(const lap_batch *b, int32_t which, int64_t *value)
     case LAP_BSTAT_UNITS: *value = b->n_units; return LAP_OK;
     case LAP_BSTAT_RERUNS: *value = b->reruns; return LAP_OK;
     case LAP_BSTAT_GRAPH_CAPTURES: *value = b->captures; return LAP_OK;
+    case LAP_BSTAT_BRANCHES: *value = b->ran_branches; return LAP_OK;
     default: return LAP_ERR_INVALID_ARG;
     }
 }

@@ -557,6 +557,8 @@ lap_status lap_get_stat(lap_graph *g, int32_t stat, int64_t *value)
     case LAP_STAT_SLOTS: *value = (int64_t)slots_for(g, choose_kernel(g), 0); return LAP_OK;
     case LAP_STAT_KERNEL: *value = choose_kernel(g); return LAP_OK;
     case LAP_STAT_LAST_KERNEL: *value = g->used_kernel; return LAP_OK;
+    case LAP_STAT_LAST_FORM: *value = g->used_form; return LAP_OK;
+    case LAP_STAT_TREE_FORM: *value = g->tree_form; return LAP_OK;
     case LAP_STAT_FALLBACKS: {
         lap_status s = resolve_pending(g);
         if (s != LAP_OK) return s;
@@ -694,6 +696,7 @@ static lap_status sample_chunk(lap_graph *g, uint64_t n_samples, uint64_t seed, 
     g->seed = seed;
     g->seed_set = true;
     g->used_kernel = kernel;
+    g->used_form = !cta ? kernel : plan.small ? LAP_FORM_SMALL : LAP_FORM_BLOCK;
 
     LapSampleLaunch p;
     memset(&p, 0, sizeof(p));
@@ -1064,6 +1067,7 @@ static lap_status spantree_block(lap_graph *g, LapSampleLaunch &p, uint64_t n_sa
     if (h.ovf_count) return LAP_OK;                  // these trees again, with the other kernel
     // (After a status bit the trees are undefined; the caller reports it.)
     *c = m;
+    g->tree_form = LAP_FORM_BLOCK;
     t->trees = p.tree_out;
     t->tree_stride = 1;
     return h.status ? spantree_failed(g, h.status) : LAP_OK;
@@ -1085,6 +1089,7 @@ static lap_status spantree_wide(lap_graph *g, LapSampleLaunch &p, uint64_t n_sam
     p.slot_epoch = g->d_slot_epoch;
     p.flags = LAP_SAMPLE_ONE_PER_LANE | LAP_SAMPLE_WILSON_ONLY;
     LAP_CUDA(g, lap_launch_sample(p, g->stream));
+    g->tree_form = LAP_FORM_WIDE;
     t->trees = reinterpret_cast<const uint32_t *>(g->ws);
     t->tree_stride = 2;
     return LAP_OK;

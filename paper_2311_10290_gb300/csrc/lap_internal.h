@@ -417,6 +417,7 @@ struct lap_graph {
     uint32_t stack_cap = 0;                 // 0: default, about 16 sqrt(n)
     int last_kernel = 0;                    // layout the workspace currently holds
     int used_kernel = 0;                    // kernel of the last lap_sample call (LAP_STAT_LAST_KERNEL)
+    int used_form = 0, tree_form = 0;       // LAP_STAT_LAST_FORM, LAP_STAT_TREE_FORM
     bool compact_disabled = false;          // set after a compact launch overflowed
     int64_t fallbacks = 0;
 
