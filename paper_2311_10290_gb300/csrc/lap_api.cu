@@ -279,9 +279,10 @@ lap_status launch_cta(lap_graph *g, LapSampleLaunch &p, LapCtaPlan &pl)
     LAP_CUDA(g, cudaStreamWaitEvent(g->side, g->fork, 0));
     cudaError_t e = lap_launch_cta_walks(p, pl, g->side);
     if (e == cudaSuccess) e = lap_launch_cta_wilson(p, pl, g->stream);
+    // Joined on errors too: walks that have been launched use the workspace.
     const cudaError_t f = cudaEventRecord(g->joined, g->side);
-    if (e == cudaSuccess) e = f;
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(g->stream, g->joined, 0);
+    const cudaError_t h = f == cudaSuccess ? cudaStreamWaitEvent(g->stream, g->joined, 0) : f;
+    if (e == cudaSuccess) e = h;
     if (e != cudaSuccess) return cuda_fail(g, e, "sampler launch (kernel 3)");
     return LAP_OK;
 }
