@@ -78,9 +78,11 @@ typedef enum {
                                   draw disjoint sample-id ranges whose counts add up exactly. */
     LAP_OPT_KERNEL = 5,        /* 0 = automatic: kernel 3 with the automatic number of walkers where
                                   its state fits (a bit per node in an SM's shared memory, about
-                                  n < 1.7 million, and 20 n + 1.2 MB of workspace for one sample);
-                                  else kernel 3 with 8 or 16 walkers for calls of at most 320
-                                  samples per SM (1024 when the graph's arrays exceed 96 MB) on
+                                  n < 1.7 million, and 20 n + 1.2 MB of workspace for one sample)
+                                  and is the faster one by an estimate from n, 2m / d_v, the
+                                  call's samples and the workspace (calls of many samples on small
+                                  graphs are not); else kernel 3 with 8 or 16 walkers for calls of at
+                                  most 320 samples per SM (1024 when the graph's arrays exceed 96 MB) on
                                   graphs of at least 2^14 nodes, else kernel 2 when n < 2^27, else
                                   kernel 1.
                                   1 = 8-byte state per node.

@@ -254,8 +254,18 @@ bool choose_cta(const lap_graph *g, uint64_t n_samples, LapCtaPlan *pl)
 {
     if (g->walkers || g->compact_disabled || !g->ws) return false;
     if (g->kernel_opt != 0 && g->kernel_opt != LAP_KERNEL_GROUP) return false;
-    return lap_cta_plan(g->n, g->arcs, g->root_degree, g->max_degree, n_samples, g->slots_opt, g->ws_bytes, g->num_sms, g->paths_opt != 0, g->cv1 || g->cv2,
-                        g->d_arcs != nullptr, pl);
+    const bool paths = g->paths_opt != 0, cv = g->cv1 || g->cv2;
+    if (!lap_cta_plan(g->n, g->arcs, g->root_degree, g->max_degree, n_samples, g->slots_opt, g->ws_bytes, g->num_sms, paths, cv,
+                      g->d_arcs != nullptr, pl))
+        return false;
+    // (The several-walkers kernel, which takes calls of few samples on graphs of 2^14 nodes
+    // on otherwise, is behind at every size measured.)
+    const int other = g->kernel_opt ? LAP_KERNEL_GROUP : choose_kernel(g, n_samples);
+    if (other == LAP_KERNEL_GROUP) return true;
+    uint64_t lanes = slots_for(g, other, n_samples);
+    if (lanes > 2048ull * (uint64_t)g->num_sms) lanes = 2048ull * (uint64_t)g->num_sms;
+    return lap_cta_estimate(g->n, g->arcs, g->root_degree, n_samples, *pl) <=
+           lap_lanes_estimate(g->n, g->arcs, g->root_degree, n_samples, lanes, other == LAP_KERNEL_WIDE, paths, cv);
 }
 
 lap_status launch_cta(lap_graph *g, LapSampleLaunch &p, LapCtaPlan &pl)

@@ -197,6 +197,12 @@ struct LapCtaPlan {
 };
 bool lap_cta_plan(int32_t n, int64_t arcs, int32_t root_degree, int32_t max_degree, uint64_t count, uint64_t slots_opt, uint64_t ws_bytes, int num_sms, bool paths,
                   bool cv, bool pack, LapCtaPlan *out);
+// Estimates in microseconds, for the choice between a plan and a lane per sample
+// (sampler_cta.cu): the plan's launch, and kernel 1 (wide) or 2 with `lanes` samples in
+// flight.
+double lap_cta_estimate(int32_t n, int64_t arcs, int32_t root_degree, uint64_t count, const LapCtaPlan &pl);
+double lap_lanes_estimate(int32_t n, int64_t arcs, int32_t root_degree, uint64_t count, uint64_t lanes, bool wide,
+                          bool paths, bool cv);
 // Fills in the plan's pointers: ws: its first words_bytes() hold zeros, or
 // words of this layout under other tags.
 void lap_cta_bind(LapSampleLaunch &p, LapCtaPlan &pl, void *ws, const unsigned long long *arcs, uint32_t tag_base);

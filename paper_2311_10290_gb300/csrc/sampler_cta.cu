@@ -41,6 +41,44 @@ bool lap_cta_plan(int32_t n, int64_t arcs, int32_t root_degree, int32_t max_degr
     return true;
 }
 
+// A lane per sample costs the time of one run for every round of `lanes` samples,
+// little more per sample until the lanes fill the memory system; a CTA per sample ends a
+// run ten to thirty times sooner, but a few hundred run at a time.  So few samples go to
+// the CTAs, and many samples of small graphs, of graphs with long first walks (f = 2m / d_v
+// steps) or in a workspace that holds few CTAs' state to the lanes.  Fitted to 454
+// measured pairs: n from 300 to 100,000, f from 17 to 37,000, 64 to 10^6 samples,
+// workspaces from 1 MB to 17 GB; in 442 of them the choice by these estimates is within 1.1
+// of the faster side, in the others within 1.5.  Both sides (lane / CTA kernel):
+// Barabasi-Albert, 1000 nodes, 10^4 samples 4.2 / 2.4 ms, 10^5 samples 7.9 / 22 ms;
+// 8000 nodes, 10^5 samples 60 / 59 ms; Erdos-Renyi, 10^4 nodes, 10^4 samples 107 / 54 ms,
+// 4 10^4 samples 128 / 129 ms, 10^5 samples 185 / 289 ms.
+double lap_lanes_estimate(int32_t n, int64_t arcs, int32_t root_degree, uint64_t count, uint64_t lanes, bool wide,
+                          bool paths, bool cv)
+{
+    const double f = (double)arcs / (double)(root_degree > 0 ? root_degree : 1), c = (double)count;
+    const double walk = 15.0 * (paths ? (cv ? 2.2 : 1.6) : cv ? 1.3 : 1.0);
+    const double rounds = lanes < count ? c / (double)(lanes > 0 ? lanes : 1) : 1.0;
+    const double each = wide ? 0.25e-3 * n + 0.25e-3 * f : 0.056e-3 * n + 0.1e-3 * f;
+    return rounds * (3.2 * n + walk * f) + c * each;
+}
+
+double lap_cta_estimate(int32_t n, int64_t arcs, int32_t root_degree, uint64_t count, const LapCtaPlan &pl)
+{
+    const double f = (double)arcs / (double)(root_degree > 0 ? root_degree : 1), c = (double)count;
+    if (pl.small) {
+        // 0.9 us per step of a sample, or the issue rate.
+        const double steps = 1.4 * n + 3.0 * f, lat = 0.9 / (double)pl.lane.slots;
+        return 1.5 * (n + 2.0 * f) + c * steps * (lat > 0.08e-3 ? lat : 0.08e-3);
+    }
+    // A first walk without an early table costs more; fewer CTAs than the SMs hold leave
+    // each of them faster.
+    const LapBlockPlan &b = pl.block;
+    const double early = b.b.part < count || b.b.early_count >= count ? 1.0 : (double)b.b.early_count / c;
+    const double each = 0.17 + 0.045e-3 * n + f * (early * 0.5e-3 * (1.0 + 1e-5 * n) + (1.0 - early) * 2.2e-3);
+    const double rounds = c > (double)b.slots ? c / (double)b.slots : 1.0, starved = 0.8 * (double)b.walk_ctas * rounds;
+    return 6.5 * f + each * (c > starved ? c : starved);
+}
+
 void lap_cta_bind(LapSampleLaunch &p, LapCtaPlan &pl, void *ws_ptr, const unsigned long long *arcs, uint32_t tag_base)
 {
     uint8_t *ws = reinterpret_cast<uint8_t *>(ws_ptr);
