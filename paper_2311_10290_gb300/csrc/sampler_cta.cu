@@ -47,9 +47,9 @@ bool lap_cta_plan(int32_t n, int64_t arcs, int32_t root_degree, int32_t max_degr
 // little more per sample until the lanes fill the memory system; a CTA per sample ends a
 // run ten to thirty times sooner, but a few hundred run at a time.  So few samples go to
 // the CTAs, and many samples of small graphs, of graphs with long first walks (f = 2m / d_v
-// steps) or in a workspace that holds few CTAs' state to the lanes.  Fitted to 454
+// steps) or in a workspace that holds few CTAs' state to the lanes.  Fitted to 462
 // measured pairs: n from 300 to 100,000, f from 17 to 37,000, 64 to 10^6 samples,
-// workspaces from 1 MB to 17 GB; in 444 of them the choice by these estimates is within 1.1
+// workspaces from 1 MB to 17 GB; in 449 of them the choice by these estimates is within 1.1
 // of the faster side, in the others within 1.5.  Both sides (lane / CTA kernel):
 // Barabasi-Albert, 1000 nodes, 10^4 samples 4.2 / 2.4 ms, 10^5 samples 7.9 / 22 ms;
 // 8000 nodes, 10^5 samples 60 / 59 ms; Erdos-Renyi, 10^4 nodes, 10^4 samples 107 / 54 ms,
@@ -72,14 +72,16 @@ double lap_cta_estimate(int32_t n, int64_t arcs, int32_t root_degree, uint64_t c
         const double steps = 1.4 * n + 3.0 * f, lat = 0.9 / (double)pl.lane.slots;
         return 1.5 * (n + 2.0 * f) + c * steps * (lat > 0.08e-3 ? lat : 0.08e-3);
     }
-    // Every part of the call waits for its longest first walk; a first walk without an
-    // early table costs more; fewer CTAs than the SMs hold leave each of them faster.
+    // Every part of the call waits for the longest of its samples' first walks (an early
+    // table each), whose lengths scatter like exponential ones; a first walk without a table
+    // costs the CTAs more; fewer CTAs than the SMs hold leave each of them faster.
     const LapBlockPlan &b = pl.block;
-    const double early = b.b.part < count || b.b.early_count >= count ? 1.0 : (double)b.b.early_count / c;
-    const double each = 0.17 + 0.045e-3 * n + f * (early * 0.5e-3 * (1.0 + 1e-5 * n) + (1.0 - early) * 2.2e-3);
+    const bool in_parts = b.b.part < count;
+    const double part = in_parts ? (double)b.b.part : c, parts = ceil(c / part);
+    const double early = in_parts || b.b.early_count >= count ? 1.0 : (double)b.b.early_count / c;
     const double rounds = c > (double)b.slots ? c / (double)b.slots : 1.0, starved = 0.8 * (double)b.walk_ctas * rounds;
-    const double parts = b.b.part < count ? ceil(c / (double)b.b.part) : 1.0;
-    return 6.5 * f * parts + each * (c > starved ? c : starved);
+    return 0.75 * f * log(part + 1.0) * parts + c * early * f * 0.5e-3 * (1.0 + 1e-5 * n) +
+           (c > starved ? c : starved) * (0.17 + 0.045e-3 * n + (1.0 - early) * 2.2e-3 * f);
 }
 
 void lap_cta_bind(LapSampleLaunch &p, LapCtaPlan &pl, void *ws_ptr, const unsigned long long *arcs, uint32_t tag_base)

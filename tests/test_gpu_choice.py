@@ -24,6 +24,7 @@ GRAPHS = {"ba": lambda n: I.ba(n, 5, seed=1), "er": lambda n: I.er(n, 10 / n, se
     ("er", 1000, 10000, 2 << 30, 0, LAP_FORM_SMALL), ("er", 2000, 100000, 4 << 30, 0, LAP_FORM_COMPACT),
     ("er", 5000, 5000, 8 << 30, 0, LAP_FORM_BLOCK), ("er", 5000, 100000, 8 << 30, 0, LAP_FORM_COMPACT),
     ("er", 16000, 10000, 16 << 30, 0, LAP_FORM_BLOCK), ("er", 20000, 100000, 16 << 30, 0, LAP_FORM_COMPACT),
+    ("er", 10000, 1000, 64 << 20, 0, LAP_FORM_BLOCK), ("er", 15000, 300, 30 << 20, 0, LAP_FORM_BLOCK),
     ("rmat", 0, 40000, 16 << 30, 0, LAP_FORM_BLOCK),
     ("ba", 1400, 10000, 80 << 20, 1, LAP_FORM_COMPACT), ("ba", 500, 2000, 5 << 20, 0, LAP_FORM_COMPACT)])
 def test_choice(family, n, samples, ws, paths, form):
