@@ -81,7 +81,8 @@ typedef enum {
                                   n < 1.7 million, and 20 n + 1.2 MB of workspace for one sample)
                                   and is the faster one by an estimate from n, 2m / d_v, the
                                   call's samples and the workspace (calls of many samples on small
-                                  graphs are not); else kernel 3 with 8 or 16 walkers for calls of at
+                                  graphs are not; small graphs with long walks need 6 n bytes of
+                                  workspace for a sample, 17 n with LAP_OPT_PATHS = 1); else kernel 3 with 8 or 16 walkers for calls of at
                                   most 320 samples per SM (1024 when the graph's arrays exceed 96 MB) on
                                   graphs of at least 2^14 nodes, else kernel 2 when n < 2^27, else
                                   kernel 1.

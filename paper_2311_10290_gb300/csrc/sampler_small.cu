@@ -189,6 +189,14 @@ bool lap_small_plan(int32_t n, int64_t arcs, uint64_t count, uint64_t slots_opt,
     uint64_t want = count;
     if (slots_opt && slots_opt < want) want = slots_opt;
     if (want == 0) want = 1;
+    // What the workspace holds: a sample's stack and words of nodes drawn often, with
+    // loop-included paths 3/8 of a walk's words (a sample's two walks take at most that share
+    // of its run's time) and one walk's at least.
+    const uint64_t entries = (nn + 7ull) & ~7ull, slot_bytes = 2ull * entries + 4ull * nn;
+    const uint64_t path_bytes = paths ? 8ull * nn : 0ull, least = 512ull + path_bytes;
+    const uint64_t hold = ws_bytes > least ? (ws_bytes - least) / (slot_bytes + 3ull * path_bytes / 8ull) : 0ull;
+    if (hold == 0) return false;
+    if (want > hold) want = hold;
     uint64_t per_sm = (want + num_sms - 1) / num_sms;
     if (per_sm > 16ull * 32ull) per_sm = 16ull * 32ull;
     // The graph's copy stays if it leaves room for the samples the call can use,
@@ -209,11 +217,10 @@ bool lap_small_plan(int32_t n, int64_t arcs, uint64_t count, uint64_t slots_opt,
     pl.smem = (pl.local ? graph : 0ull) + warps * lanes * per_lane;
     // Workspace: path words of the loop-included paths, the stacks, the words of
     // nodes drawn often.
-    const uint64_t entries = (nn + 7ull) & ~7ull;
-    const uint64_t slots = pl.blocks * warps * lanes;
-    const uint64_t stacks = (2ull * entries + 4ull * nn) * slots + 512ull;
-    const uint64_t path_bytes = paths ? 8ull * nn : 0ull;
-    if (stacks + path_bytes > ws_bytes) return false;
+    pl.slots = pl.blocks * warps * lanes;
+    if (pl.slots > hold) pl.slots = hold;
+    if (slots_opt && slots_opt < pl.slots) pl.slots = slots_opt;
+    const uint64_t stacks = slot_bytes * pl.slots + 512ull;
     pl.b.path_lanes = 0;
     if (paths) {
         pl.b.path_lanes = (ws_bytes - stacks) / path_bytes;
@@ -221,10 +228,9 @@ bool lap_small_plan(int32_t n, int64_t arcs, uint64_t count, uint64_t slots_opt,
     }
     pl.words_bytes = pl.b.path_lanes * path_bytes;
     pl.stack_offset = (pl.words_bytes + 255ull) & ~255ull;
-    pl.many_offset = pl.stack_offset + 2ull * entries * slots;
+    pl.many_offset = pl.stack_offset + 2ull * entries * pl.slots;
     pl.bytes = pl.words_bytes + stacks;
     pl.b.stack_entries = entries;
-    pl.slots = slots_opt && slots_opt < slots ? slots_opt : slots;
     *out = pl;
     return true;
 }
