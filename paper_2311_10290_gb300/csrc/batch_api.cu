@@ -23,6 +23,8 @@
 #include "lap_batch.h"
 #include "lap_internal.h"
 
+constexpr int kBranches = 16;             // of a captured run; each has a stream for its walks beside it
+
 struct lap_batch {
     int device = 0;
     int num_sms = 0;
@@ -63,8 +65,8 @@ struct lap_batch {
 
     cudaStream_t stream = nullptr;
     cudaStream_t cap_stream = nullptr;
-    cudaStream_t branch_streams[20] = {};            // branches of a captured run; re-runs
-    cudaEvent_t branch_done[20] = {};
+    cudaStream_t branch_streams[2 * kBranches] = {}; // branches of a captured run, and their walks; re-runs
+    cudaEvent_t branch_done[2 * kBranches] = {};
     std::vector<int32_t> root_degree, max_degree;
     cudaEvent_t fork = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -100,7 +102,6 @@ struct lap_batch {
 namespace {
 
 thread_local std::string g_batch_error = "no error";
-constexpr int kBranches = 16, kWalkBranches = 4;
 constexpr int kRerunStreams = 8;                     // of the branch streams
 constexpr uint64_t kPackBytes = 96ull << 20;         // packed arcs that stay in L2
 
@@ -133,7 +134,7 @@ void free_batch(lap_batch *b)
 {
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
-    for (int k = 0; k < kBranches + kWalkBranches; ++k) {
+    for (int k = 0; k < 2 * kBranches; ++k) {
         if (b->branch_streams[k]) cudaStreamDestroy(b->branch_streams[k]);
         if (b->branch_done[k]) cudaEventDestroy(b->branch_done[k]);
     }
@@ -318,7 +319,7 @@ LapBatchLaunch make_launch(const lap_batch *b, uint64_t seed, uint64_t lanes, ui
 lap_status ensure_branches(lap_batch *b)
 {
     if (!b->fork) B_CUDA(b, cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming));
-    for (int k = 0; k < kBranches + kWalkBranches; ++k) {
+    for (int k = 0; k < 2 * kBranches; ++k) {
         if (!b->branch_streams[k]) B_CUDA(b, cudaStreamCreateWithFlags(&b->branch_streams[k], cudaStreamNonBlocking));
         if (!b->branch_done[k]) B_CUDA(b, cudaEventCreateWithFlags(&b->branch_done[k], cudaEventDisableTiming));
     }
@@ -421,7 +422,7 @@ cudaError_t launch_branches(lap_batch *b, Branches &br, const LapBatchLaunch &re
     stamp_kernel<<<1, 1, 0, cs>>>(&b->d_ctl->t0);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaEventRecord(b->fork, cs);
-    for (int t = 0; t < kBranches + kWalkBranches && e == cudaSuccess; ++t)
+    for (int t = 0; t < 2 * kBranches && e == cudaSuccess; ++t)
         e = cudaStreamWaitEvent(b->branch_streams[t], b->fork, 0);
     const int32_t m = (int32_t)br.order.size();
     std::vector<LapSampleLaunch> launches((size_t)m);
@@ -444,17 +445,12 @@ cudaError_t launch_branches(lap_batch *b, Branches &br, const LapBatchLaunch &re
         p.ovf_ids = b->d_rerun_ids + (uint64_t)g * samples;
         lap_cta_bind(p, br.plan[(size_t)k], ws, b->packed[(size_t)g] ? b->d_arcs + b->csr_arc_off[(size_t)g] : nullptr, 0);
     }
-    // The absorbed walks, longest expected first (2m / d_v steps).
-    std::vector<int32_t> by_length((size_t)m);
-    std::iota(by_length.begin(), by_length.end(), 0);
-    auto length = [&](int32_t k) {
-        const size_t g = (size_t)br.order[(size_t)k];
-        return (double)b->arcs[g] / (double)b->root_degree[g];
-    };
-    std::stable_sort(by_length.begin(), by_length.end(), [&](int32_t x, int32_t y) { return length(x) > length(y); });
-    for (int32_t j = 0; j < m && e == cudaSuccess; ++j) {
-        const int32_t k = by_length[(size_t)j];
-        cudaStream_t st = b->branch_streams[kBranches + j % kWalkBranches];
+    // The absorbed walks, beside each branch and in its order, so that a graph's are done
+    // about when its Wilson runs are.  (On four streams, longest first, the small graphs of
+    // a batch of 120 ended with its longest walks: median 253 ms of 305 with the smallest
+    // first, now 35 of 294; the run's time is the same or less.)
+    for (int32_t k = 0; k < m && e == cudaSuccess; ++k) {
+        cudaStream_t st = b->branch_streams[kBranches + br.branch[(size_t)k]];
         e = lap_launch_cta_walks(launches[(size_t)k], br.plan[(size_t)k], st);
         if (e != cudaSuccess) break;
         stamp_kernel<<<1, 1, 0, st>>>(b->d_tdone + br.order[(size_t)k]);
@@ -472,7 +468,7 @@ cudaError_t launch_branches(lap_batch *b, Branches &br, const LapBatchLaunch &re
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && !br.rest.empty()) e = lap_launch_batch(rest, false, cs);
-    for (int t = 0; t < kBranches + kWalkBranches; ++t) {      // joined on errors too: the capture must end
+    for (int t = 0; t < 2 * kBranches; ++t) {      // joined on errors too: the capture must end
         const cudaError_t f = cudaEventRecord(b->branch_done[t], b->branch_streams[t]);
         const cudaError_t h = cudaStreamWaitEvent(cs, b->branch_done[t], 0);
         if (e == cudaSuccess) e = f != cudaSuccess ? f : h;

@@ -1,0 +1,31 @@
+"""LAP_BOPT_ORDER in a run on branches: with the smallest graphs first, most graphs are done
+long before the batch is (their absorbed walks do not queue behind the longest ones), and
+the smallest ones long before the largest."""
+import numpy as np
+import pytest
+
+from paper_2311_10290_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+from paper_2311_10290_gb300.lap import LAP_BOPT_ORDER, LAP_BSTAT_BRANCHES, LapBatch  # noqa: E402
+
+
+def test_smallest_first_completes_small_graphs_early():
+    graphs = I.batch_graphs(I.batch_spec(60, 1000, 50000, seed0=3))
+    n = np.array([g.n for g in graphs])
+    B = LapBatch([(g.row_ptr, g.col) for g in graphs], workspace_bytes=4 << 30)
+    try:
+        B.set_option(LAP_BOPT_ORDER, 1)
+        for _ in range(2):
+            B.run(512, 5)
+            B.sync()
+        c = np.asarray(B.completion())
+        assert B.stat(LAP_BSTAT_BRANCHES) == len(graphs)
+    finally:
+        B.close()
+    small = n <= np.quantile(n, 0.25)
+    assert c[small].min() < 0.1 * c.max()
+    assert np.median(c) < 0.4 * c.max()
+    assert np.median(c[small]) < np.median(c[~small])
