@@ -339,6 +339,27 @@ struct Branches {
     std::vector<int> branch;             // of order[k]
     std::vector<LapCtaPlan> plan;        // of order[k]
 };
+// The persistent sampler's time for the graphs in `which`, in microseconds: the longest run,
+// or the lanes' share of all runs, and what a sample adds while the lanes fill the memory
+// system.
+double persistent_estimate(const lap_batch *b, const std::vector<int32_t> &which, uint64_t samples, uint64_t lanes)
+{
+    double longest = 0.0, runs = 0.0, each = 0.0;
+    for (int32_t k : which) {
+        const size_t g = (size_t)k;
+        const double run = lap_lanes_estimate(b->n[g], b->arcs[g], b->root_degree[g], 1, 1, false, false, false);
+        longest = std::max(longest, run);
+        runs += run * (double)samples;
+        each += lap_lanes_estimate(b->n[g], b->arcs[g], b->root_degree[g], samples, samples, false, false, false) - run;
+    }
+    return std::max(longest, runs / (double)std::max<uint64_t>(lanes, 1)) + each;
+}
+
+// False, too, where the persistent sampler is the faster one for all graphs: many small
+// graphs, many samples of small graphs (300 graphs of 500 to 2000 nodes, 64 samples 10 ms
+// persistent, 16 ms on branches, 1000 samples 30 / 72 ms; 64 Erdos-Renyi graphs of 1000
+// nodes, 4096 samples 41 / 122 ms; 120 graphs of up to 60,000 nodes, 512 samples 688 /
+// 280 ms).
 bool plan_branches(const lap_batch *b, uint64_t samples, Branches *out)
 {
     if (samples > LAP_TAGS) return false;
@@ -379,6 +400,26 @@ bool plan_branches(const lap_batch *b, uint64_t samples, Branches *out)
     // The persistent sampler's slots take the first half, if it has graphs.
     const uint64_t base = br.rest.empty() ? 0ull : (b->ws_bytes / 2ull) & ~255ull;
     if (m == 0 || (base && base < slot_bytes_of(b))) return false;
+    const uint64_t lanes = lanes_for(b, samples, b->lanes_opt, nullptr);
+    std::vector<int32_t> every((size_t)b->G);
+    std::iota(every.begin(), every.end(), 0);
+    const double persistent = persistent_estimate(b, every, samples, lanes);
+    const double rest = br.rest.empty() ? 0.0 : persistent_estimate(b, br.rest, samples, lanes / 2);
+    // With all the workspace they ask for: a branch runs its graphs one after the other, each
+    // some 200 us of launches at least, and what fills the SMs adds up.  (The sum takes
+    // branches for less overlapped than they are: on 20 batches, those with 1.5 and more were
+    // faster persistent, those below 1.45 on branches.)
+    const double limit = 1.45 * persistent;
+    double longest = 0.0, serial = 0.0, work = 0.0;
+    for (int32_t k : br.order) {
+        const size_t g = (size_t)k;
+        plan(k, 1ull << 50);
+        const double alone = lap_cta_estimate(b->n[g], b->arcs[g], b->root_degree[g], samples, pl);
+        longest = std::max(longest, alone);
+        serial += (alone + 200.0) / (double)std::min<int32_t>(kBranches, m);
+        work += lap_cta_work(b->n[g], b->arcs[g], b->root_degree[g], samples, pl, b->num_sms);
+    }
+    if (std::max(longest, serial) + work + rest > limit) return false;
     br.plan.resize((size_t)m);
     for (br.count = std::min<int32_t>(kBranches, m); br.count >= 1; br.count /= 2) {
         std::vector<uint64_t> load((size_t)br.count, 0), want((size_t)br.count, 0);
@@ -401,6 +442,15 @@ bool plan_branches(const lap_batch *b, uint64_t samples, Branches *out)
             br.plan[(size_t)k] = pl;
         }
         if (!ok) continue;
+        // With the shares they get: the slowest branch, whose estimate alone is about twice what
+        // it takes beside the others.
+        std::vector<double> alone((size_t)br.count, 0.0);
+        for (int32_t k = 0; k < m; ++k) {
+            const size_t g = (size_t)br.order[(size_t)k];
+            alone[(size_t)br.branch[(size_t)k]] +=
+                200.0 + lap_cta_estimate(b->n[g], b->arcs[g], b->root_degree[g], samples, br.plan[(size_t)k]);
+        }
+        if (0.5 * *std::max_element(alone.begin(), alone.end()) + rest > limit) return false;
         *out = br;
         return true;
     }

@@ -201,6 +201,8 @@ bool lap_cta_plan(int32_t n, int64_t arcs, int32_t root_degree, int32_t max_degr
 // (sampler_cta.cu): the plan's launch, and kernel 1 (wide) or 2 with `lanes` samples in
 // flight.
 double lap_cta_estimate(int32_t n, int64_t arcs, int32_t root_degree, uint64_t count, const LapCtaPlan &pl);
+// The part of it in which the launch fills the SMs: what it adds to other launches beside it.
+double lap_cta_work(int32_t n, int64_t arcs, int32_t root_degree, uint64_t count, const LapCtaPlan &pl, int num_sms);
 double lap_lanes_estimate(int32_t n, int64_t arcs, int32_t root_degree, uint64_t count, uint64_t lanes, bool wide,
                           bool paths, bool cv);
 // Fills in the plan's pointers: ws: its first words_bytes() hold zeros, or

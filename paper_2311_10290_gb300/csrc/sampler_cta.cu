@@ -84,6 +84,18 @@ double lap_cta_estimate(int32_t n, int64_t arcs, int32_t root_degree, uint64_t c
            (c > starved ? c : starved) * (0.17 + 0.045e-3 * n + (1.0 - early) * 2.2e-3 * f);
 }
 
+double lap_cta_work(int32_t n, int64_t arcs, int32_t root_degree, uint64_t count, const LapCtaPlan &pl, int num_sms)
+{
+    const double f = (double)arcs / (double)(root_degree > 0 ? root_degree : 1), c = (double)count;
+    if (pl.small) {
+        // A CTA has an SM's shared memory to itself.
+        const double steps = 1.4 * n + 3.0 * f, waves = ceil(c / (double)pl.lane.slots);
+        const double share = (double)pl.lane.blocks / (double)num_sms, issue = c * steps * 0.08e-3;
+        return share * waves * steps * 0.9 > issue ? share * waves * steps * 0.9 : issue;
+    }
+    return c * (0.17 + 0.045e-3 * n + f * 0.5e-3 * (1.0 + 1e-5 * n));
+}
+
 void lap_cta_bind(LapSampleLaunch &p, LapCtaPlan &pl, void *ws_ptr, const unsigned long long *arcs, uint32_t tag_base)
 {
     uint8_t *ws = reinterpret_cast<uint8_t *>(ws_ptr);
