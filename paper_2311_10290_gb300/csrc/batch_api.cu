@@ -409,7 +409,12 @@ bool plan_branches(const lap_batch *b, uint64_t samples, Branches *out)
     // some 200 us of launches at least, and what fills the SMs adds up.  (The sum takes
     // branches for less overlapped than they are: on 20 batches, those with 1.5 and more were
     // faster persistent, those below 1.45 on branches.)
-    const double limit = 1.45 * persistent;
+    // With smallest first or the caller's order, what counts is when the graphs are complete,
+    // and graphs on branches would wait for the registers of the persistent sampler beside
+    // them (all 512 graphs of the uneven recipe, 4096 samples, smallest first: half complete
+    // after 32.5 s of 41.5, persistent alone 1.9 s of 50.5; 60 graphs of up to 100,000 nodes,
+    // 3000 samples 300 of 1393 ms, 180 of 1098): there branches have to be ahead for certain.
+    const double limit = (b->order_opt != 0 && !br.rest.empty() ? 0.77 : 1.45) * persistent;
     double longest = 0.0, serial = 0.0, work = 0.0;
     for (int32_t k : br.order) {
         const size_t g = (size_t)k;

@@ -29,3 +29,23 @@ def test_smallest_first_completes_small_graphs_early():
     assert c[small].min() < 0.1 * c.max()
     assert np.median(c) < 0.4 * c.max()
     assert np.median(c[small]) < np.median(c[~small])
+
+
+def test_order_is_kept_where_both_samplers_would_run():
+    """Enough samples of graphs with long first walks to fill the persistent sampler: graphs
+    on branches would wait for it, so it takes them all when an order is asked for."""
+    graphs = I.batch_graphs(I.batch_spec(60, 1000, 50000, seed0=3))
+    B = LapBatch([(g.row_ptr, g.col) for g in graphs], workspace_bytes=16 << 30)
+    try:
+        branches, done = [], []
+        for order in (0, 1):
+            B.set_option(LAP_BOPT_ORDER, order)
+            for _ in range(2):
+                B.run(5000, 5)
+                B.sync()
+            branches.append(B.stat(LAP_BSTAT_BRANCHES))
+            done.append(np.asarray(B.completion()))
+    finally:
+        B.close()
+    assert 0 < branches[0] < len(graphs) and branches[1] == 0
+    assert np.median(done[1]) < 0.4 * done[1].max()
