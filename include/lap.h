@@ -131,7 +131,7 @@ typedef enum {
                                   the popped cycles, so every node's draws and the tree, do not
                                   depend on the order in which walkers find them), then one runs
                                   the uniform-start walk and one the pi-start walk. */
-    LAP_OPT_PATH_START = 8     /* -1 (default): the first absorbed walk (or loop-included path) of
+    LAP_OPT_PATH_START = 8,    /* -1 (default): the first absorbed walk (or loop-included path) of
                                   each sample starts at a uniform draw (Alg. 2).  s in [0, n): it
                                   starts at node s, so its passes of u have mean d_u (L_v^{-1})_{su}
                                   (Section 4.2, "v-absorbed walk" and "loop-erased walk" lemmas)
@@ -141,6 +141,10 @@ typedef enum {
                                   lap_rw_betweenness, the CV ECC) are then refused
                                   (LAP_ERR_INVALID_ARG); Wilson counts and lap_kemeny are unchanged.
                                   Only before the first sample after lap_set_root. */
+    LAP_OPT_WITHDRAW = 10      /* a check of the re-runs: w > 0 makes the form of kernel 3 with a CTA per
+                                  sample withdraw every w-th sample of a launch (at its start,
+                                  before its sweeps and at its end in turn), as it does a sample
+                                  without progress; counts are the same.  0 (default): none */
 } lap_option;
 
 /* Statistics for lap_get_stat. */

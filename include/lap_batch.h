@@ -47,7 +47,8 @@ typedef enum {
                             both samplers to the persistent one) */
     LAP_BOPT_BLOCK = 4,  /* threads per block; 0 = automatic */
     LAP_BOPT_STACK = 5,  /* loop-erased path capacity per lane; 0 = 16 sqrt(largest n), at least 1024 */
-    LAP_BOPT_PATHS = 6   /* LAP_OPT_PATHS for every graph of the batch (0 default, 1 loop-included paths) */
+    LAP_BOPT_PATHS = 6,  /* LAP_OPT_PATHS for every graph of the batch (0 default, 1 loop-included paths) */
+    LAP_BOPT_WITHDRAW = 7 /* LAP_OPT_WITHDRAW for the graphs on branches (0 default) */
 } lap_batch_option;
 
 /* Statistics for lap_batch_stat. */

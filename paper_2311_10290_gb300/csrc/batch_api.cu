@@ -72,7 +72,7 @@ struct lap_batch {
     cudaGraphExec_t exec = nullptr;
     bool key_valid = false;
     uint64_t key_samples = 0, key_seed = 0, key_lanes = 0;
-    uint32_t key_claim = 0, key_stack = 0, key_paths = 0;
+    uint32_t key_claim = 0, key_stack = 0, key_paths = 0, key_withdraw = 0;
     int key_order = -1, key_block = -1;
     bool key_cta = false;                // the captured run may take the branches ...
     bool exec_cta = false;               // ... and does ...
@@ -86,6 +86,7 @@ struct lap_batch {
     int block_opt = 0;
     uint32_t stack_opt = 0;
     uint32_t paths_opt = 0;
+    uint32_t withdraw_opt = 0;
 
     uint64_t omega = 0;
     uint64_t seed = 0;
@@ -499,6 +500,7 @@ cudaError_t launch_branches(lap_batch *b, Branches &br, const LapBatchLaunch &re
         p.ustart_dev = &b->d_graphs[g].ustart;
         p.ovf_ids = b->d_rerun_ids + (uint64_t)g * samples;
         lap_cta_bind(p, br.plan[(size_t)k], ws, b->packed[(size_t)g] ? b->d_arcs + b->csr_arc_off[(size_t)g] : nullptr, 0);
+        br.plan[(size_t)k].block.b.withdraw = b->withdraw_opt;
     }
     // The absorbed walks, beside each branch and in its order, so that a graph's are done
     // about when its Wilson runs are.  (On four streams, longest first, the small graphs of
@@ -594,6 +596,7 @@ lap_status capture(lap_batch *b, uint64_t samples, uint64_t seed, uint64_t lanes
     b->key_block = block;
     b->key_stack = stack_cap_of(b);
     b->key_paths = b->paths_opt;
+    b->key_withdraw = b->withdraw_opt;
     ++b->captures;
     return LAP_OK;
 }
@@ -1015,6 +1018,10 @@ lap_status lap_batch_set_option(lap_batch *b, int32_t option, int64_t value)
         if (b->paths_opt != (uint32_t)value) b->meta_dirty = true;   // the slot layout changes
         b->paths_opt = (uint32_t)value;
         return LAP_OK;
+    case LAP_BOPT_WITHDRAW:
+        if (value > 0x7FFFFFFF) return bfail(b, LAP_ERR_INVALID_ARG, "withdraw must be below 2^31");
+        b->withdraw_opt = (uint32_t)value;
+        return LAP_OK;
     case LAP_BOPT_STACK:
         if (value != 0 && (value < 16 || value > (1 << 26) || (value & 3))) return bfail(b, LAP_ERR_INVALID_ARG, "stack capacity must be 0 or a multiple of 4 in [16, 2^26]");
         if ((uint32_t)value != b->stack_opt) b->meta_dirty = true;
@@ -1075,7 +1082,7 @@ lap_status lap_batch_run(lap_batch *b, uint64_t samples_per_graph, uint64_t seed
     const uint32_t claim = b->claim_opt;
     if (!b->key_valid || !b->exec || b->key_samples != samples_per_graph || b->key_seed != seed || b->key_lanes != lanes ||
         b->key_claim != claim || b->key_order != b->order_opt || b->key_block != block || b->key_stack != stack_cap_of(b) ||
-        b->key_paths != b->paths_opt || b->key_cta != default_options(b)) {
+        b->key_paths != b->paths_opt || b->key_withdraw != b->withdraw_opt || b->key_cta != default_options(b)) {
         s = capture(b, samples_per_graph, seed, lanes, claim, block);
         if (s != LAP_OK) return s;
     }

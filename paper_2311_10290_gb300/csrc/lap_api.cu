@@ -285,6 +285,7 @@ lap_status launch_cta(lap_graph *g, LapSampleLaunch &p, LapCtaPlan &pl)
     LAP_CUDA(g, cudaMemsetAsync(&g->d_acc->claim, 0, sizeof(unsigned int), g->stream));
     LAP_CUDA(g, cudaMemsetAsync(&g->d_acc->walk_claim, 0, sizeof(unsigned int), g->stream));
     lap_cta_bind(p, pl, g->ws, g->d_arcs, tag);
+    pl.block.b.withdraw = g->withdraw_opt;
     LAP_CUDA(g, cudaEventRecord(g->fork, g->stream));
     LAP_CUDA(g, cudaStreamWaitEvent(g->side, g->fork, 0));
     cudaError_t e = lap_launch_cta_walks(p, pl, g->side);
@@ -533,6 +534,10 @@ lap_status lap_set_option(lap_graph *g, int32_t option, int64_t value)
         if (value != 0 && (value < 16 || value > (1 << 22))) return fail(g, LAP_ERR_INVALID_ARG, "stack capacity must be 0 or in [16, 2^22]");
         g->stack_cap = (uint32_t)value;
         g->last_kernel = 0;
+        return LAP_OK;
+    case LAP_OPT_WITHDRAW:
+        if (value > 0x7FFFFFFF) return fail(g, LAP_ERR_INVALID_ARG, "withdraw must be below 2^31");
+        g->withdraw_opt = (uint32_t)value;
         return LAP_OK;
     case LAP_OPT_BLOCK:
         if (value != 0 && (value % 32 != 0 || value > 256)) return fail(g, LAP_ERR_INVALID_ARG, "block must be 0 or a multiple of 32 up to 256");
@@ -1077,6 +1082,7 @@ static lap_status spantree_block(lap_graph *g, LapSampleLaunch &p, uint64_t n_sa
     p.count = (uint32_t)m;
     p.tree_out = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(g->ws) + half);
     lap_cta_bind(p, pl, g->ws, g->d_arcs, 0u);
+    pl.block.b.withdraw = g->withdraw_opt;
     LAP_CUDA(g, lap_launch_cta_wilson(p, pl, g->stream));
     LapDevAcc h;
     LAP_CUDA(g, cudaMemcpyAsync(&h, g->d_st_acc, sizeof(h), cudaMemcpyDeviceToHost, g->stream));

@@ -156,6 +156,7 @@ struct LapBlockLaunch {
     uint32_t early_cap;                       // path entries of a sample
     uint32_t part;                            // samples of the call that are run at a time
     uint32_t ovf_cap;                         // entries of LapSampleLaunch::ovf_ids
+    uint32_t withdraw;                        // LAP_OPT_WITHDRAW
     uint32_t *early, *early_stacks, *early_pops;
 };
 struct LapBlockPlan {
@@ -417,6 +418,7 @@ struct lap_graph {
 
     uint64_t step_limit = 0;                // 0: default
     uint64_t slots_opt = 0;
+    uint32_t withdraw_opt = 0;              // LAP_OPT_WITHDRAW
     int block_opt = 0;
     int kernel_opt = 0;                     // 0 auto, LAP_KERNEL_WIDE, LAP_KERNEL_COMPACT, LAP_KERNEL_GROUP
     int walkers = 0;                        // LAP_OPT_WALKERS (kernel 3; 0 = automatic)

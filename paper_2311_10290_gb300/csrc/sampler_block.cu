@@ -84,6 +84,7 @@ constexpr uint32_t cInflight = 28;    // two-node pops under way
 constexpr uint32_t cIn = 32;          // sweeps: entries of the list read ...
 constexpr uint32_t cTake = 36;        // ... taken so far ...
 constexpr uint32_t cOut = 40;         // ... and written
+constexpr uint32_t cGiveUp = 44;      // LAP_OPT_WITHDRAW: withdraw the sample at its start (1), before the sweeps (2), at its end (3)
 constexpr uint32_t kCtlBytes = 48;
 constexpr uint32_t kQueue = 64;        // nodes a warp collects for a batch of 32 arrows
 constexpr uint32_t kNoArrow = 0xFFFFFFFFu;
@@ -397,7 +398,9 @@ __global__ void __launch_bounds__(1024, 1) lewalk_block_kernel(LapSampleLaunch p
             sts(ctl + cCursor, 0u);
             sts(ctl + cExcl, 0u);
             sts(ctl + cInflight, 0u);
-            sts(ctl + cStatus, p.step_limit < n - 1u || e > pop_limit ? kStLimit : 0u);
+            const uint32_t give_up = b.withdraw && q % b.withdraw == 0u ? 1u + q / b.withdraw % 3u : 0u;
+            sts(ctl + cGiveUp, give_up);
+            sts(ctl + cStatus, p.step_limit < n - 1u || e > pop_limit ? kStLimit : give_up == 1u ? kStWithdraw : 0u);
         }
         group_sync();
         if (early) {
@@ -755,7 +758,7 @@ __global__ void __launch_bounds__(1024, 1) lewalk_block_kernel(LapSampleLaunch p
         }
 
         group_sync();
-        if (stage || goal == n || lds(ctl + cDone) >= n || lds(ctl + cStatus)) break;
+        if (stage || goal == n || lds(ctl + cDone) >= n || lds(ctl + cStatus) || lds(ctl + cGiveUp) == 2u) break;
         {
         uint32_t added = 0;
         // The node's arrow leads to w in the tree, seen with k = ku.
@@ -918,7 +921,7 @@ __global__ void __launch_bounds__(1024, 1) lewalk_block_kernel(LapSampleLaunch p
         }
 
         group_sync();
-        const unsigned st = lds(ctl + cStatus);
+        const unsigned st = lds(ctl + cStatus) | (lds(ctl + cGiveUp) ? kStWithdraw : 0u);
         if (st & kStLimit) bad |= LAP_DEV_STEP_LIMIT;
         if (st & kStOverflow) bad |= LAP_DEV_K_OVERFLOW;
         if (st & kStWithdraw) {

@@ -29,6 +29,7 @@ LAP_OPT_STEP_LIMIT, LAP_OPT_SLOTS, LAP_OPT_BLOCK, LAP_OPT_CURSOR, LAP_OPT_KERNEL
 LAP_OPT_PATHS = 7
 LAP_OPT_PATH_START = 8
 LAP_OPT_WALKERS = 9
+LAP_OPT_WITHDRAW = 10
 LAP_STAT_SLOTS, LAP_STAT_KERNEL, LAP_STAT_FALLBACKS, LAP_STAT_LAST_KERNEL = 1, 2, 3, 4
 LAP_STAT_LAST_FORM, LAP_STAT_TREE_FORM = 5, 6
 LAP_FORM_WIDE, LAP_FORM_COMPACT, LAP_FORM_GROUP, LAP_FORM_BLOCK, LAP_FORM_SMALL = 1, 2, 3, 4, 5
@@ -37,6 +38,7 @@ LAP_MLP_TCGEN05, LAP_MLP_MMA_SYNC = 0, 1
 LAP_BOPT_LANES, LAP_BOPT_CLAIM, LAP_BOPT_ORDER, LAP_BOPT_BLOCK, LAP_BOPT_STACK, LAP_BOPT_PATHS = 1, 2, 3, 4, 5, 6
 LAP_BSTAT_LANES, LAP_BSTAT_CLAIM, LAP_BSTAT_UNITS, LAP_BSTAT_RERUNS, LAP_BSTAT_GRAPH_CAPTURES = 1, 2, 3, 4, 5
 LAP_BSTAT_BRANCHES = 6
+LAP_BOPT_WITHDRAW = 7
 
 
 class LapError(RuntimeError):
