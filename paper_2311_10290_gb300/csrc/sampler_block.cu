@@ -84,7 +84,6 @@ constexpr uint32_t cInflight = 28;    // two-node pops under way
 constexpr uint32_t cIn = 32;          // sweeps: entries of the list read ...
 constexpr uint32_t cTake = 36;        // ... taken so far ...
 constexpr uint32_t cOut = 40;         // ... and written
-constexpr uint32_t cGiveUp = 44;      // LAP_OPT_WITHDRAW: withdraw the sample at its start (1), before the sweeps (2), at its end (3)
 constexpr uint32_t kCtlBytes = 48;
 constexpr uint32_t kQueue = 64;        // nodes a warp collects for a batch of 32 arrows
 constexpr uint32_t kNoArrow = 0xFFFFFFFFu;
@@ -330,8 +329,16 @@ __global__ void __launch_bounds__(128) lewalk_early_kernel(LapSampleLaunch p, La
     b.early_pops[q] = pops;
 }
 
-// One sample per CTA at a time.
-template <bool CV, bool PACK>
+// LAP_OPT_WITHDRAW: whether sample q is withdrawn at its start (when 0), before its sweeps
+// (1) or at its end (2).
+__device__ __forceinline__ bool give_up(const LapBlockLaunch &b, uint32_t q, uint32_t when)
+{
+    return q % b.withdraw == 0u && q / b.withdraw % 3u == when;
+}
+
+// One sample per CTA at a time.  CHECK: with LAP_OPT_WITHDRAW (in the kernel of other calls
+// its tests, once per sample, cost 3 % on 10^6 nodes, 205 -> 212 ms).
+template <bool CV, bool PACK, bool CHECK>
 __global__ void __launch_bounds__(1024, 1) lewalk_block_kernel(LapSampleLaunch p, LapBlockLaunch b)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -398,9 +405,8 @@ __global__ void __launch_bounds__(1024, 1) lewalk_block_kernel(LapSampleLaunch p
             sts(ctl + cCursor, 0u);
             sts(ctl + cExcl, 0u);
             sts(ctl + cInflight, 0u);
-            const uint32_t give_up = b.withdraw && q % b.withdraw == 0u ? 1u + q / b.withdraw % 3u : 0u;
-            sts(ctl + cGiveUp, give_up);
-            sts(ctl + cStatus, p.step_limit < n - 1u || e > pop_limit ? kStLimit : give_up == 1u ? kStWithdraw : 0u);
+            sts(ctl + cStatus, p.step_limit < n - 1u || e > pop_limit ? kStLimit : 0u);
+            if (CHECK && give_up(b, q, 0u)) reds_or(ctl + cStatus, kStWithdraw);
         }
         group_sync();
         if (early) {
@@ -758,7 +764,7 @@ __global__ void __launch_bounds__(1024, 1) lewalk_block_kernel(LapSampleLaunch p
         }
 
         group_sync();
-        if (stage || goal == n || lds(ctl + cDone) >= n || lds(ctl + cStatus) || lds(ctl + cGiveUp) == 2u) break;
+        if (stage || goal == n || lds(ctl + cDone) >= n || lds(ctl + cStatus) || (CHECK && give_up(b, q, 1u))) break;
         {
         uint32_t added = 0;
         // The node's arrow leads to w in the tree, seen with k = ku.
@@ -920,8 +926,9 @@ __global__ void __launch_bounds__(1024, 1) lewalk_block_kernel(LapSampleLaunch p
         }
         }
 
+        if (CHECK && j == 0 && (give_up(b, q, 1u) || give_up(b, q, 2u))) reds_or(ctl + cStatus, kStWithdraw);
         group_sync();
-        const unsigned st = lds(ctl + cStatus) | (lds(ctl + cGiveUp) ? kStWithdraw : 0u);
+        const unsigned st = lds(ctl + cStatus);
         if (st & kStLimit) bad |= LAP_DEV_STEP_LIMIT;
         if (st & kStOverflow) bad |= LAP_DEV_K_OVERFLOW;
         if (st & kStWithdraw) {
@@ -989,11 +996,13 @@ uint32_t bits_for(uint64_t x)          // smallest b with x < 2^b
 constexpr uint64_t kSmemMax = 227ull << 10;
 uint64_t align16(uint64_t x) { return (x + 15ull) & ~15ull; }
 
-const void *kernel_for(bool cv, bool pack)
+template <bool CHECK>
+const void *kernel_of(bool cv, bool pack)
 {
-    if (cv) return pack ? (const void *)lewalk_block_kernel<true, true> : (const void *)lewalk_block_kernel<true, false>;
-    return pack ? (const void *)lewalk_block_kernel<false, true> : (const void *)lewalk_block_kernel<false, false>;
+    if (cv) return pack ? (const void *)lewalk_block_kernel<true, true, CHECK> : (const void *)lewalk_block_kernel<true, false, CHECK>;
+    return pack ? (const void *)lewalk_block_kernel<false, true, CHECK> : (const void *)lewalk_block_kernel<false, false, CHECK>;
 }
+const void *kernel_for(bool cv, bool pack, bool check = false) { return check ? kernel_of<true>(cv, pack) : kernel_of<false>(cv, pack); }
 
 template <bool CV, bool PACK>
 void launch_early(const LapSampleLaunch &p, const LapBlockLaunch &b, unsigned blocks, cudaStream_t st)
@@ -1148,7 +1157,11 @@ cudaError_t lap_launch_sample_block(const LapSampleLaunch &all, const LapBlockPl
 {
     if (all.count == 0 || pl.slots == 0) return cudaSuccess;
     const bool cv = all.cv_h1 || all.cv_h2, pack = pl.b.arcs != nullptr;
-    const void *kernel = kernel_for(cv, pack);
+    const void *kernel = kernel_for(cv, pack, pl.b.withdraw != 0u);
+    if (pl.b.withdraw) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+        if (e != cudaSuccess) return e;
+    }
     for (uint32_t done = 0; done < all.count; done += pl.b.part) {
         LapSampleLaunch p = all;
         LapBlockLaunch b = pl.b;
