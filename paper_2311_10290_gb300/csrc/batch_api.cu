@@ -41,6 +41,7 @@ struct lap_batch {
     int2 *d_rowinfo = nullptr;
     unsigned long long *d_arcs = nullptr;            // packed arcs (lap_launch_pack_arcs) of the graphs with packed[g]
     std::vector<char> packed;
+    std::vector<int64_t> pack_off;                   // and where a graph's begin
     unsigned long long *d_rep1 = nullptr, *d_cnt2 = nullptr, *d_scratch = nullptr;
     double *d_ldiag = nullptr, *d_ecc = nullptr, *d_red = nullptr;
     LapBatchGraph *d_graphs = nullptr;
@@ -499,7 +500,7 @@ cudaError_t launch_branches(lap_batch *b, Branches &br, const LapBatchLaunch &re
         p.num_sms = b->num_sms;
         p.ustart_dev = &b->d_graphs[g].ustart;
         p.ovf_ids = b->d_rerun_ids + (uint64_t)g * samples;
-        lap_cta_bind(p, br.plan[(size_t)k], ws, b->packed[(size_t)g] ? b->d_arcs + b->csr_arc_off[(size_t)g] : nullptr, 0);
+        lap_cta_bind(p, br.plan[(size_t)k], ws, b->packed[(size_t)g] ? b->d_arcs + b->pack_off[(size_t)g] : nullptr, 0);
         br.plan[(size_t)k].block.b.withdraw = b->withdraw_opt;
     }
     // The absorbed walks, beside each branch and in its order, so that a graph's are done
@@ -887,15 +888,18 @@ lap_status lap_batch_create(int32_t n_graphs, const int32_t *n, const int32_t *c
     for (size_t g = 0; g < G && e == cudaSuccess; ++g)
         if (b->src[g] == (int32_t)g)
             e = lap_launch_rowinfo(d_row_ptr + b->csr_node_off[g] + (int64_t)g, n[g], b->d_rowinfo + b->csr_node_off[g], st);
-    // Packed arcs where a graph's stay in L2 (an allocation that fails leaves the
-    // plain columns).
+    // Packed arcs where a graph's stay in L2, shared like the CSRs (an allocation that
+    // fails leaves the plain columns).
     b->packed.assign(G, 0);
-    bool any_packed = false;
+    b->pack_off.assign(G, 0);
+    int64_t pack_arcs = 0;
     for (size_t g = 0; g < G; ++g) {
+        const size_t s = (size_t)b->src[g];
         b->packed[g] = n[g] <= (1 << 21) && 8ull * (uint64_t)b->arcs[g] <= kPackBytes;
-        any_packed = any_packed || b->packed[g];
+        b->pack_off[g] = s == g ? pack_arcs : b->pack_off[s];
+        if (b->packed[g] && s == g) pack_arcs += b->arcs[g];
     }
-    if (e == cudaSuccess && any_packed && balloc(&b->d_arcs, (size_t)b->csr_arcs) != cudaSuccess) {
+    if (e == cudaSuccess && pack_arcs && balloc(&b->d_arcs, (size_t)pack_arcs) != cudaSuccess) {
         cudaGetLastError();
         b->d_arcs = nullptr;
         b->packed.assign(G, 0);
@@ -903,7 +907,7 @@ lap_status lap_batch_create(int32_t n_graphs, const int32_t *n, const int32_t *c
     for (size_t g = 0; g < G && e == cudaSuccess; ++g)
         if (b->packed[g] && b->src[g] == (int32_t)g)
             e = lap_launch_pack_arcs(b->d_rowinfo + b->csr_node_off[g], b->d_col + b->csr_arc_off[g], n[g], b->arcs[g],
-                                     b->d_arcs + b->csr_arc_off[g], st);
+                                     b->d_arcs + b->pack_off[g], st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cudaFree(d_row_ptr);
     d_row_ptr = nullptr;
