@@ -165,26 +165,35 @@ int choose_kernel(const lap_graph *g, uint64_t n_samples = 0)
     return LAP_KERNEL_COMPACT;
 }
 
+// Makes sure a workspace exists: without a lent one, what `kernel` can use, at most half of
+// the free memory.
+lap_status allocate_workspace(lap_graph *g, int kernel)
+{
+    if (g->ws) return LAP_OK;
+    const uint64_t per_slot = slot_bytes_of(g, kernel);
+    size_t free_b = 0, total_b = 0;
+    LAP_CUDA(g, cudaMemGetInfo(&free_b, &total_b));
+    uint64_t want = (uint64_t)free_b / 2;
+    uint64_t cap = per_slot * (uint64_t)g->num_sms * 2048ull;
+    if (want > cap) want = cap;
+    want = (want / 256) * 256;
+    if (want < per_slot) return fail(g, LAP_ERR_OOM, "not enough device memory for one Wilson state");
+    cudaError_t e = cudaMalloc(&g->ws, want);
+    if (e != cudaSuccess) { cudaGetLastError(); g->ws = nullptr; return fail(g, LAP_ERR_OOM, "workspace allocation failed"); }
+    g->ws_bytes = want;
+    g->ws_owned = true;
+    g->ws_zeroed = false;
+    return LAP_OK;
+}
+
 // Makes sure a workspace exists and holds the layout of `kernel`, zeroed
 // when the layout changed (epoch bits then read "stale" everywhere).
 lap_status ensure_workspace(lap_graph *g, int kernel)
 {
     const uint64_t per_slot = slot_bytes_of(g, kernel);
     g->blk_clean = 0;
-    if (!g->ws) {
-        size_t free_b = 0, total_b = 0;
-        LAP_CUDA(g, cudaMemGetInfo(&free_b, &total_b));
-        uint64_t want = (uint64_t)free_b / 2;
-        uint64_t cap = per_slot * (uint64_t)g->num_sms * 2048ull;
-        if (want > cap) want = cap;
-        want = (want / 256) * 256;
-        if (want < per_slot) return fail(g, LAP_ERR_OOM, "not enough device memory for one Wilson state");
-        cudaError_t e = cudaMalloc(&g->ws, want);
-        if (e != cudaSuccess) { cudaGetLastError(); g->ws = nullptr; return fail(g, LAP_ERR_OOM, "workspace allocation failed"); }
-        g->ws_bytes = want;
-        g->ws_owned = true;
-        g->ws_zeroed = false;
-    }
+    const lap_status s = allocate_workspace(g, kernel);
+    if (s != LAP_OK) return s;
     const uint64_t slots = g->ws_bytes / per_slot;
     if (slots == 0) return fail(g, LAP_ERR_OOM, "workspace smaller than one sample's state");
     if (kernel == LAP_KERNEL_GROUP) {
@@ -705,7 +714,7 @@ static lap_status sample_chunk(lap_graph *g, uint64_t n_samples, uint64_t seed, 
     if (n_samples == 0) return LAP_OK;
     if ((s = resolve_pending(g)) != LAP_OK) return s;
     LapCtaPlan plan;
-    if (!g->ws && (s = ensure_workspace(g, LAP_KERNEL_GROUP)) != LAP_OK) return s;
+    if ((s = allocate_workspace(g, choose_kernel(g, n_samples))) != LAP_OK) return s;
     const bool cta = choose_cta(g, n_samples, &plan);
     const int kernel = cta ? LAP_KERNEL_GROUP : choose_kernel(g, n_samples);
     if (!cta && (s = ensure_workspace(g, kernel)) != LAP_OK) return s;
@@ -1128,7 +1137,7 @@ lap_status lap_spantree_sample(lap_graph *g, uint64_t n_samples, uint64_t seed)
     if (n_samples == 0) return LAP_OK;
     if ((s = resolve_pending(g)) != LAP_OK) return s;      // the workspace is about to be reused
     if ((s = spantree_prepare(g)) != LAP_OK) return s;
-    if (!g->ws && (s = ensure_workspace(g, LAP_KERNEL_WIDE)) != LAP_OK) return s;
+    if ((s = allocate_workspace(g, LAP_KERNEL_WIDE)) != LAP_OK) return s;
     g->st_seed = seed;
     g->st_seed_set = true;
     const uint64_t limit = g->step_limit ? g->step_limit : default_step_limit(g->n);
