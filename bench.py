@@ -130,6 +130,7 @@ def parse():
                     help="measure the random 1-byte read+write ceiling the sampler is compared with (0: skip)")
     ap.add_argument("--extra-cv", type=int, default=0,
                     help="also measure the control variate against plain on the extra workloads (1: on)")
+    ap.add_argument("--details", default="", help="file that receives the whole result (JSON)")
     return ap.parse_args()
 
 
@@ -1581,6 +1582,49 @@ def run_reference(args, rank, world):
             "e2e": {"value": value, "unit": "walk steps/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
 
 
+# ------------------------------------------------------------ output
+
+# What the one line on stdout holds.  Readers of it keep a few kilobytes; with the studies of
+# a full run the result is ten times that, so these go to stderr and to --details.
+LINE_KEYS = ("impl", "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better",
+             "scaling", "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "roofline",
+             "cpu_baseline", "walk_steps", "merged_estimate")
+LINE_BYTES = 3400
+
+
+def studies_summary(res):
+    """Seconds (and samples) of the studies, by name."""
+    out = {}
+
+    def add(name, d):
+        if isinstance(d, dict):
+            s = {k: d[k] for k in ("omega", "omega_extrapolated", "gpu_seconds", "seconds", "trees_per_s")
+                 if isinstance(d.get(k), (int, float))}
+            if s:
+                out[name] = {k: round(v, 5) if isinstance(v, float) else v for k, v in s.items()}
+
+    add("time_to_accuracy", res.get("time_to_accuracy"))
+    for r in res.get("time_to_accuracy_large") or []:
+        for form in ("plain", "paths", "cv", "cvpaths"):
+            add("%s/%s" % (r.get("workload", "?"), form), r.get(form))
+    add("spantree", res.get("spantree"))
+    add("spantree_time_to_accuracy", (res.get("spantree") or {}).get("time_to_accuracy"))
+    add("batched", res.get("batched"))
+    return out
+
+
+def stdout_line(res):
+    """The result's line for stdout: the measurement itself, and the studies in brief as far
+    as they fit."""
+    line = {k: res[k] for k in LINE_KEYS if k in res}
+    brief = studies_summary(res)
+    if brief:
+        line["studies"] = brief
+        while line["studies"] and len(json.dumps(line)) > LINE_BYTES:
+            line["studies"].popitem()
+    return json.dumps(line)
+
+
 def main():
     args = parse()
     rank = int(os.environ.get("RANK", "0"))
@@ -1590,7 +1634,11 @@ def main():
     else:
         res = run_ours(args, rank, world)
     if rank == 0 and res is not None:
-        print(json.dumps(res), flush=True)
+        if args.details:
+            with open(args.details, "w") as f:
+                json.dump(res, f)
+        print("[bench] %s" % json.dumps({k: v for k, v in res.items() if k not in LINE_KEYS}), file=sys.stderr, flush=True)
+        print(stdout_line(res), flush=True)
 
 
 if __name__ == "__main__":
