@@ -1033,13 +1033,16 @@ def spantree_measurement(torch, LapGraph, g, v, args):
         b.record()
         torch.cuda.synchronize()
         t = a.elapsed_time(b) / 1e3
+        from paper_2311_10290_gb300.lap import LAP_STAT_TREE_FORM
+        sampler = KERNEL_NAMES[G.stat(LAP_STAT_TREE_FORM)]
         _, _, kc = G.spantree_estimates()
     finally:
         G.close()
     return {"workload": g.name, "trees": args.spantree_trees, "seconds": t, "trees_per_s": args.spantree_trees / t,
             "kemeny_estimate": kc, "time_to_accuracy": spantree_tta(torch, LapGraph),
-            "note": "trees: 8-byte Wilson kernel, one tree per lane, then one CTA per tree for the flow sums "
-                    "(children, levels, subtree sizes, preorder intervals, BFS-path sums)"}
+            "sampler": sampler,
+            "note": "trees by `sampler`, then one CTA per tree for the flow sums (subtree sizes and degree sums from "
+                    "the leaves up, preorder intervals by pointer jumping, BFS-path sums)"}
 
 
 # ------------------------------------------------------------ studies (batched runtime)
@@ -1208,11 +1211,12 @@ def extra_workload(torch, LapGraph, name, args, params):
 def batched_measurement(torch, args):
     """Uneven batch: graphs of the recipe in inputs.batch_spec (ER, BA, R-MAT;
     n log-uniform in [1e3, 1e6]; average degree in [4, 32]; own root each),
-    all sampled in one persistent CUDA-graph launch with autotuned lanes and
-    claim size.  Times one run of `batched_samples` samples per graph after a
+    all sampled in one CUDA-graph launch: on branches, by the persistent sampler with
+    autotuned lanes and claim size, or both.  Times one run of `batched_samples` samples per graph after a
     warm-up run of 1/16 of them."""
     from paper_2311_10290_gb300 import inputs
-    from paper_2311_10290_gb300.lap import LAP_BOPT_ORDER, LAP_BSTAT_CLAIM, LAP_BSTAT_LANES, LAP_BSTAT_RERUNS, LapBatch
+    from paper_2311_10290_gb300.lap import (LAP_BOPT_ORDER, LAP_BSTAT_BRANCHES, LAP_BSTAT_CLAIM, LAP_BSTAT_LANES,
+                                            LAP_BSTAT_RERUNS, LapBatch)
     t0 = time.perf_counter()
     spec = inputs.batch_spec(count=args.batched_graphs, n_hi=args.batched_nmax)
     graphs = inputs.batch_graphs(spec)
@@ -1249,7 +1253,7 @@ def batched_measurement(torch, args):
                          "completion_seconds": {"p50": float(np.percentile(done, 50)),
                                                 "p99": float(np.percentile(done, 99)),
                                                 "max": float(done.max()), "min": float(done.min())},
-                         "reruns": B.stat(LAP_BSTAT_RERUNS)})
+                         "reruns": B.stat(LAP_BSTAT_RERUNS), "graphs_on_branches": B.stat(LAP_BSTAT_BRANCHES)})
         kc = B.kemeny()
         wilson = uwalk = piwalk = inserts = 0
         for j, g in enumerate(graphs):
@@ -1277,15 +1281,18 @@ def batched_measurement(torch, args):
             "walk_steps": {"wilson": wilson, "uniform_walk": uwalk, "pi_walk": piwalk},
             "value": steps / t_total, "unit": "walk steps/s",
             "completion_seconds": best["completion_seconds"], "order": best["order"], "runs": runs,
+            # (lanes, claim and autotune: of the persistent sampler)
             "lanes": B.stat(LAP_BSTAT_LANES), "claim": B.stat(LAP_BSTAT_CLAIM), "reruns": best["reruns"],
             "autotune": [{"lanes": a, "claim": c, "walk_steps_per_s": round(r, 1)} for a, c, r in table],
             "autotune_seconds": round(t_tune, 2), "generate_seconds": round(t_gen, 2),
             "create_seconds": round(t_create, 2),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                         "kernel": "lewalk_batch_kernel (+ batched finalize, in one CUDA graph)",
+                         "kernel": "%d graphs by lewalk_block_kernel and lewalk_small_kernel on branches, %d by "
+                                   "lewalk_batch_kernel (+ batched finalize, in one CUDA graph)"
+                                   % (best["graphs_on_branches"], len(graphs) - best["graphs_on_branches"]),
                          "peak_kind": peak_kind},
             "kemeny_first_graphs": [round(float(x), 3) for x in kc[:4]],
-            "note": "seconds: CUDA graph launch (resets, persistent sampler, finalize of every graph) to results "
+            "note": "seconds: CUDA graph launch (resets, sampling, finalize of every graph) to results "
                     "ready, re-runs of withdrawn samples included; completion: from the sampler's start to each "
                     "graph's last sample; top-level value/completion: the faster of `runs` (same samples, same "
                     "counts: only the unit order differs)",
