@@ -110,8 +110,9 @@ typedef enum {
                                   left 255 times by one loop-included path) are withdrawn and
                                   re-run with kernel 1.
                                   Counts are identical with every kernel. */
-    LAP_OPT_STACK = 6,         /* loop-erased path capacity per sample (kernel 2) or walker (kernel 3); 0 = default
-                                  (16 sqrt(n) rounded up to a power of two, at least 1024) */
+    LAP_OPT_STACK = 6,         /* loop-erased path capacity per sample (kernel 2) or walker (kernel 3 with a
+                                  number of walkers; its other forms size their paths themselves); 0 =
+                                  default (16 sqrt(n) rounded up to a power of two, at least 1024) */
     LAP_OPT_PATHS = 7,         /* 0 (default): the uniform-start and pi-start v-absorbed walks take
                                   their own draws, as Alg. 2 and Alg. 4 print them.  1: they are the
                                   loop-included paths of the sample's own Wilson stacks (Section 4.2,

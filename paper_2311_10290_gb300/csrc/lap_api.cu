@@ -4,9 +4,9 @@
 #include <atomic>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
-#include <vector>
 
 #include "lap_internal.h"
 
@@ -458,12 +458,17 @@ lap_status lap_graph_create(int32_t n, const int32_t *row_ptr, const int32_t *co
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hub_count, &g->d_acc->claim, sizeof(hub_count), cudaMemcpyDeviceToHost, g->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
     if (e == cudaSuccess && hub_count) {
-        std::vector<int32_t> ids(hub_count);
+        std::unique_ptr<int32_t[]> ids(new (std::nothrow) int32_t[hub_count]);
+        if (!ids) {
+            free_all(g);
+            delete g;
+            return fail(nullptr, LAP_ERR_OOM, "host allocation failed");
+        }
         const size_t bytes = sizeof(int32_t) * hub_count;
-        e = cudaMemcpyAsync(ids.data(), g->d_hubs, bytes, cudaMemcpyDeviceToHost, g->stream);
+        e = cudaMemcpyAsync(ids.get(), g->d_hubs, bytes, cudaMemcpyDeviceToHost, g->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
-        std::sort(ids.begin(), ids.end());
-        if (e == cudaSuccess) e = cudaMemcpyAsync(g->d_hubs, ids.data(), bytes, cudaMemcpyHostToDevice, g->stream);
+        std::sort(ids.get(), ids.get() + hub_count);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(g->d_hubs, ids.get(), bytes, cudaMemcpyHostToDevice, g->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
     }
     g->hubs = LapHubs{g->d_hubs, (int32_t)hub_count};

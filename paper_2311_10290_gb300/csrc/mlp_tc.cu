@@ -204,9 +204,10 @@ __device__ __forceinline__ float warp_sum(float x)
 
 // ------------------------------------------------------------ forward
 
-// Bound by instruction issue (about 400 per warp and tile, of which 64 x 2 biases and
-// the conversions are most) once a tile's three round trips to the tensor core are
-// hidden.  One group per CTA, four CTAs per SM, rows loaded when their tile began
+// Bound by the shared-memory pipe (75 % busy: the operand stores and bias reads of the
+// epilogues) and by the waits of a tile, which eight tiles per SM hide in part: about 540
+// instructions per warp and tile take 44 % of the issue slots, the tensor pipe is 14 %
+// busy, DRAM 11 %.  One group per CTA, four CTAs per SM, rows loaded when their tile began
 // and 64 accumulators held per thread: 45 us on 1,000,003 rows; now 35 us.
 constexpr int kGroups = 4;
 constexpr uint32_t fSW1 = 0;                            // B  [64 x 16]   W1
@@ -384,7 +385,7 @@ __global__ void __launch_bounds__(kThreads * kGroups, 2)
 
 // Loss and gradient: G and loss accumulate the batch's MSE gradient and loss.
 // Bound by the chain of one tile (six round trips to the tensor core) where a batch
-// has no more tiles than SMs.  8192 rows: 26.7 -> 15.5 us with only the unwritten
+// has no more tiles than SMs: a warp per scheduler, which issues in 13 % of the cycles.  8192 rows: 26.7 -> 15.5 us with only the unwritten
 // operand parts cleared, the weight loads side by side, dW2 added in rows of 32
 // neighbours, and one launch to clear the outputs.
 __global__ void __launch_bounds__(kThreads, 1)

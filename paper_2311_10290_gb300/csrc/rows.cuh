@@ -10,8 +10,9 @@
 // Against one thread per row (GB300): solve of 300,000 nodes 8.5 -> 3.6 ms; root and
 // breadth-first search 1.33 -> 0.42 ms (10^6 nodes, 10^7 arcs, largest degree 4183)
 // and 11.4 -> 0.72 ms (R-MAT, 3.1 10^7 arcs, 64668); its features 69 -> 3.3 ms.
-// The solve with hubs from 256 / 512 / 2048 neighbours: 3.6 / 4.1 / 6.9 ms; with a
-// thread for rows of up to 16 / 48 / 128: 4.1 / 4.1 / 4.3 ms (hubs from 512).
+// The solve with hubs from 256 / 512 / 2048 neighbours: 3.6 / 4.1 / 6.9 ms.  Where a
+// thread's rows end matters little: up to 16 / 48 / 128 entries 4.1 / 4.1 / 4.3 ms (hubs
+// from 512).
 #pragma once
 
 #include "lap_internal.h"

@@ -38,9 +38,9 @@
 //             tree; where a pass gains little, the next one pops the two-node
 //             cycles.  No paths, no locks on the way, full warps.
 //   walkers   on the list's rest (n / 200 nodes, at least 64).
-// The sweep's line: 0.2 / 0.3 / 0.35 / 0.4 of the nodes take 91 / 84 / 78 / 79 ms on
-// the 100,000-node Barabasi-Albert graph (16384 samples), 35 / 36 / 39 / 38 ms
-// on the R-MAT graph of 31 million arcs (2048 samples).
+// The sweep's line: 0.2 / 0.28 / 0.35 / 0.4 of the nodes take 43.3 / 40.9 / 40.6 / 40.8 ms
+// on the 100,000-node Barabasi-Albert graph (8192 samples), 29.3 / 30.3 / 30.9 / 31.3 ms on
+// an R-MAT graph of 31 million arcs (1520 samples), whose columns are read from HBM.
 //
 // Memory.  Per sample in flight, in shared memory: one tree bit per node; lock
 // bits (of the nodes' low id bits); a filter bit per 2^fshift nodes, set before
@@ -52,7 +52,9 @@
 //
 // What bounds it: the walkers' dependent chain (Philox, one L2 load, shared
 // memory) while few lanes have work, and instruction issue (about 130 per
-// step) when all have.  Against a lane per sample with byte counts in HBM
+// step) when all have; the profile of 2 * 10^5 nodes has 55 % of the issue rate.  At 64
+// registers per thread (two CTAs of 480 threads on an SM) the kernel spills 104 to 120 bytes
+// in all instances.  Against a lane per sample with byte counts in HBM
 // (sampler_compact.cu), sampling only: Barabasi-Albert, 10^5 nodes, 16384
 // samples 173 -> 75 ms; 10^6 nodes, 4096 samples 750 -> 203 ms; R-MAT of 31
 // million arcs, 2048 samples 312 -> 39 ms; 2 * 10^5 nodes with control variate and
@@ -599,7 +601,7 @@ __global__ void __launch_bounds__(1024, 1) lewalk_block_kernel(LapSampleLaunch p
                 const uint32_t ou = __shfl_sync(kFull, u, o), oku = __shfl_sync(kFull, ku, o), ow = __shfl_sync(kFull, wt, o);
                 const uint2 *ob = reinterpret_cast<const uint2 *>(__shfl_sync(kFull, (unsigned long long)stk, o));
                 const uint2 *os = ob + oc;
-                                bool mayc = true;
+                bool mayc = true;
                 if (lane == 0u) {
                     mayc = atoms_cas(ctl + cExcl, 0u, 1u) == 0u;
                     __threadfence_block();
@@ -682,7 +684,7 @@ __global__ void __launch_bounds__(1024, 1) lewalk_block_kernel(LapSampleLaunch p
                 const uint32_t osp = __shfl_sync(kFull, sp, o), ou = __shfl_sync(kFull, u, o), oku = __shfl_sync(kFull, ku, o);
                 uint32_t above = __shfl_sync(kFull, wt, o);
                 const uint2 *os = reinterpret_cast<const uint2 *>(__shfl_sync(kFull, (unsigned long long)stk, o));
-                                uint32_t x0 = 0, added = 0, good = 32u;     // entry 0 is the head, entry x the x-th below it
+                uint32_t x0 = 0, added = 0, good = 32u;     // entry 0 is the head, entry x the x-th below it
                 for (; x0 <= osp; x0 += 32u) {
                     const uint32_t x = x0 + lane;
                     uint2 e = make_uint2(ou, oku);
@@ -902,7 +904,6 @@ __global__ void __launch_bounds__(1024, 1) lewalk_block_kernel(LapSampleLaunch p
             // of pass gets on.
             const bool slow = !first && out >= in - in / 8u;
             const bool hard = slow && pops && out >= in - in / 64u;
-            if (first) in = n;
             uint32_t *t = list;
             list = list2;
             list2 = t;
@@ -1044,6 +1045,12 @@ bool lap_block_plan(int32_t n, int64_t arcs, int32_t root_degree, int32_t max_de
     if (want == 0) want = 1;
     const uint64_t per_sm = (want + num_sms - 1) / num_sms;
     LapBlockLaunch &b = pl.b;
+    // Threads: as many CTAs on an SM as registers and tree bits leave room for, and the
+    // walkers a sample of that size uses.  Against the neighbouring counts: 20,000 nodes 96 /
+    // 128 / 192 threads 13.4 / 13.3 / 13.0 ms, 50,000 nodes 128 / 224 / 288: 25.9 / 24.6 /
+    // 24.7 ms, 100,000 nodes 288 / 480 / 672: 42.2 / 40.6 / 48.7 ms, 300,000 nodes 288 / 480 /
+    // 992: 73.9 / 58.5 / 59.5 ms, 10^6 nodes 480 / 992: 126 / 85.5 ms (Barabasi-Albert, 8192
+    // samples; 4096 and 1520 of the last two).  The lines lie between the measured sizes.
     pl.threads = nn < 24000 ? 128 : nn < 64000 ? 224 : nn < 400000 ? 480 : 992;
     if (per_sm * (uint64_t)(pl.threads + 32) <= 512ull) pl.threads *= 2;
     b.lmask = 8191u;
@@ -1053,11 +1060,16 @@ bool lap_block_plan(int32_t n, int64_t arcs, int32_t root_degree, int32_t max_de
     pl.smem = align16(fixed + 4ull * ((((nn - 1ull) >> fs) >> 5) + 1ull));
     if (pl.smem > kSmemMax) return false;
     b.fshift = fs;
+    // The same for every size: on the graphs above, an R-MAT graph of 31 million arcs and
+    // Erdos-Renyi graphs of 15,000 and 50,000 nodes, other values are within 1 % or slower
+    // but for walk_min 64 (3 and 5 % faster on the two graphs below 24,000 nodes) and grow 16
+    // (2 to 4 % from 50,000 nodes on); idle_min 28 costs 8 to 23 %, grow 2 up to 5 %, sweeps from
+    // 0.2 n up to 9 % (they gain 5 % on the R-MAT graph), unit_batch 1 up to 3 %.
     b.walk_min = 32u;
     b.grow = 4.0f;
     b.idle_min = 12u;
     b.pair_min = 4u;
-    b.unit_batch = nn > 200000 ? 4u : 2u;
+    b.unit_batch = 4u;
     // Paths of first walks have about sqrt(n) nodes, on sparse graphs a few times that;
     // a sample whose path does not fit ends its early phase without a tree.  (With 4096
     // entries at every size, 256 samples of Erdos-Renyi graphs of 10^6 nodes took over a

@@ -241,8 +241,6 @@ uint64_t lap_spantree_scratch_ints(int32_t n)
     return (7ull * (uint64_t)n + 1ull) & ~1ull;
 }
 
-int lap_spantree_block() { return kTB; }
-
 cudaError_t lap_launch_spantree(const LapSpanTreeLaunch &p, int blocks, cudaStream_t st)
 {
     if (p.count == 0 || blocks <= 0) return cudaSuccess;
