@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(kThreads * kGroups, 2)
 
 // Loss and gradient: G and loss accumulate the batch's MSE gradient and loss.
 // Bound by the chain of one tile (six round trips to the tensor core) where a batch
-// has no more tiles than SMs: a warp per scheduler, which issues in 13 % of the cycles.  8192 rows: 26.7 -> 15.5 us with only the unwritten
+// has no more tiles than SMs: a warp per scheduler, which issues in 13 % of the cycles.  8192 rows: 26.7 -> 17 us a call (this kernel 15.6) with only the unwritten
 // operand parts cleared, the weight loads side by side, dW2 added in rows of 32
 // neighbours, and one launch to clear the outputs.
 __global__ void __launch_bounds__(kThreads, 1)
