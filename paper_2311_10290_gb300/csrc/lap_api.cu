@@ -267,14 +267,22 @@ bool choose_cta(const lap_graph *g, uint64_t n_samples, LapCtaPlan *pl)
     if (!lap_cta_plan(g->n, g->arcs, g->root_degree, g->max_degree, n_samples, g->slots_opt, g->ws_bytes, g->num_sms, paths, cv,
                       g->d_arcs != nullptr, pl))
         return false;
-    // (The several-walkers kernel, which takes calls of few samples on graphs of 2^14 nodes
-    // on otherwise, is behind at every size measured.)
-    const int other = g->kernel_opt ? LAP_KERNEL_GROUP : choose_kernel(g, n_samples);
-    if (other == LAP_KERNEL_GROUP) return true;
-    uint64_t lanes = slots_for(g, other, n_samples);
-    if (lanes > 2048ull * (uint64_t)g->num_sms) lanes = 2048ull * (uint64_t)g->num_sms;
-    return lap_cta_estimate(g->n, g->arcs, g->root_degree, n_samples, *pl) <=
-           lap_lanes_estimate(g->n, g->arcs, g->root_degree, n_samples, lanes, other == LAP_KERNEL_WIDE, paths, cv);
+    if (g->kernel_opt) return true;
+    const int other = choose_kernel(g, n_samples);
+    const double cta = lap_cta_estimate(g->n, g->arcs, g->root_degree, n_samples, *pl);
+    uint64_t slots = slots_for(g, other, n_samples);
+    if (other == LAP_KERNEL_GROUP) {
+        // Ahead only where long first walks run in many parts: of 47 calls with 18,000 to 93,000
+        // nodes, 300 to 47,000 samples and workspaces from 0.1 to 24 GB, in 11 (Erdos-Renyi,
+        // 36,000 nodes, 37,000 samples in 2.1 GB: several walkers 1452 ms, CTAs 2526); in 9
+        // of them the estimates say so, in the others CTAs are behind by 1.17.  With 16 walkers
+        // a sample costs more (65,000 nodes, 8700 samples in 1.2 GB: 8 walkers 1523 ms, 16 walkers
+        // 1993, CTAs 1651).
+        slots = std::min<uint64_t>(slots, 160ull * (uint64_t)g->num_sms);
+        return cta <= (walkers_for(g, n_samples) == 16 ? 1.35 : 1.15) * lap_group_estimate(g->n, g->arcs, g->root_degree, n_samples, slots);
+    }
+    slots = std::min<uint64_t>(slots, 2048ull * (uint64_t)g->num_sms);
+    return cta <= lap_lanes_estimate(g->n, g->arcs, g->root_degree, n_samples, slots, other == LAP_KERNEL_WIDE, paths, cv);
 }
 
 lap_status launch_cta(lap_graph *g, LapSampleLaunch &p, LapCtaPlan &pl)

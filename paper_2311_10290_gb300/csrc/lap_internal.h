@@ -206,6 +206,8 @@ double lap_cta_estimate(int32_t n, int64_t arcs, int32_t root_degree, uint64_t c
 double lap_cta_work(int32_t n, int64_t arcs, int32_t root_degree, uint64_t count, const LapCtaPlan &pl, int num_sms);
 double lap_lanes_estimate(int32_t n, int64_t arcs, int32_t root_degree, uint64_t count, uint64_t lanes, bool wide,
                           bool paths, bool cv);
+// The same for the several-walkers kernel with 8 lanes per sample, `groups` samples in flight.
+double lap_group_estimate(int32_t n, int64_t arcs, int32_t root_degree, uint64_t count, uint64_t groups);
 // Fills in the plan's pointers: ws: its first words_bytes() hold zeros, or
 // words of this layout under other tags.
 void lap_cta_bind(LapSampleLaunch &p, LapCtaPlan &pl, void *ws, const unsigned long long *arcs, uint32_t tag_base);

@@ -64,6 +64,16 @@ double lap_lanes_estimate(int32_t n, int64_t arcs, int32_t root_degree, uint64_t
     return rounds * (3.2 * n + walk * f) + c * each;
 }
 
+// Eight lanes shorten the Wilson run, not the first walk; later rounds overlap the longest
+// runs of earlier ones.  Erdos-Renyi, 18,000 nodes, 17,300 samples in 267 MB 1508 ms (estimate
+// 1700), 57,000 nodes, 5500 samples in 552 MB 1359 (1380), 10^5 nodes, 512 samples 1258 (1060).
+double lap_group_estimate(int32_t n, int64_t arcs, int32_t root_degree, uint64_t count, uint64_t groups)
+{
+    const double f = (double)arcs / (double)(root_degree > 0 ? root_degree : 1), c = (double)count;
+    const double rounds = groups < count ? c / (double)(groups > 0 ? groups : 1) : 1.0;
+    return (0.5 + 0.5 * rounds) * (1.1 * n + 25.0 * f) + c * (0.084e-3 * n + 0.15e-3 * f);
+}
+
 double lap_cta_estimate(int32_t n, int64_t arcs, int32_t root_degree, uint64_t count, const LapCtaPlan &pl)
 {
     const double f = (double)arcs / (double)(root_degree > 0 ? root_degree : 1), c = (double)count;
@@ -80,7 +90,7 @@ double lap_cta_estimate(int32_t n, int64_t arcs, int32_t root_degree, uint64_t c
     const double part = in_parts ? (double)b.b.part : c, parts = ceil(c / part);
     const double early = in_parts || b.b.early_count >= count ? 1.0 : (double)b.b.early_count / c;
     const double rounds = c > (double)b.slots ? c / (double)b.slots : 1.0, starved = 0.8 * (double)b.walk_ctas * rounds;
-    return 0.75 * f * log(part + 1.0) * parts + c * early * f * 0.5e-3 * (1.0 + 1e-5 * n) +
+    return 0.75 * f * log(part + 1.0) * parts + c * early * f * 0.5e-3 * (1.0 + 0.5e-5 * n) +
            (c > starved ? c : starved) * (0.17 + 0.045e-3 * n + (1.0 - early) * 2.2e-3 * f);
 }
 
@@ -93,7 +103,7 @@ double lap_cta_work(int32_t n, int64_t arcs, int32_t root_degree, uint64_t count
         const double share = (double)pl.lane.blocks / (double)num_sms, issue = c * steps * 0.08e-3;
         return share * waves * steps * 0.9 > issue ? share * waves * steps * 0.9 : issue;
     }
-    return c * (0.17 + 0.045e-3 * n + f * 0.5e-3 * (1.0 + 1e-5 * n));
+    return c * (0.17 + 0.045e-3 * n + f * 0.5e-3 * (1.0 + 0.5e-5 * n));
 }
 
 void lap_cta_bind(LapSampleLaunch &p, LapCtaPlan &pl, void *ws_ptr, const unsigned long long *arcs, uint32_t tag_base)

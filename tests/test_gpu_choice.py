@@ -12,7 +12,7 @@ from paper_2311_10290_gb300 import inputs as I
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
-from paper_2311_10290_gb300.lap import (LAP_FORM_BLOCK, LAP_FORM_COMPACT, LAP_FORM_SMALL, LAP_OPT_KERNEL,  # noqa: E402
+from paper_2311_10290_gb300.lap import (LAP_FORM_BLOCK, LAP_FORM_COMPACT, LAP_FORM_GROUP, LAP_FORM_SMALL, LAP_OPT_KERNEL,  # noqa: E402
                                         LAP_OPT_PATHS, LAP_STAT_LAST_FORM, LapGraph)
 
 GRAPHS = {"ba": lambda n: I.ba(n, 5, seed=1), "er": lambda n: I.er(n, 10 / n, seed=1), "rmat": lambda n: I.rmat(13, 16, seed=1)}
@@ -25,12 +25,13 @@ GRAPHS = {"ba": lambda n: I.ba(n, 5, seed=1), "er": lambda n: I.er(n, 10 / n, se
     ("er", 5000, 5000, 8 << 30, 0, LAP_FORM_BLOCK), ("er", 5000, 100000, 8 << 30, 0, LAP_FORM_COMPACT),
     ("er", 16000, 10000, 16 << 30, 0, LAP_FORM_BLOCK), ("er", 20000, 100000, 16 << 30, 0, LAP_FORM_COMPACT),
     ("er", 10000, 1000, 64 << 20, 0, LAP_FORM_BLOCK), ("er", 15000, 300, 30 << 20, 0, LAP_FORM_BLOCK),
+    ("er", 40000, 5000, 400 << 20, 1, LAP_FORM_GROUP), ("er", 40000, 5000, 8 << 30, 1, LAP_FORM_BLOCK),
     ("rmat", 0, 40000, 16 << 30, 0, LAP_FORM_BLOCK),
     ("ba", 1400, 10000, 80 << 20, 1, LAP_FORM_COMPACT), ("ba", 500, 2000, 5 << 20, 0, LAP_FORM_COMPACT)])
 def test_choice(family, n, samples, ws, paths, form):
     g = GRAPHS[family](n)
     out = []
-    for kernel in (0, 3 if form == LAP_FORM_COMPACT else 2):
+    for kernel in (0, 2 if form in (LAP_FORM_BLOCK, LAP_FORM_SMALL) else 3):
         G = LapGraph(g.row_ptr, g.col, workspace_bytes=ws)
         try:
             G.set_option(LAP_OPT_PATHS, paths)
