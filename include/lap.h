@@ -154,7 +154,7 @@ typedef enum {
                                   the current workspace (kernel 3: groups of walkers) */
     LAP_STAT_KERNEL = 2,       /* kernel (1, 2 or 3) whose slots LAP_STAT_SLOTS and lap_workspace_query
                                   describe: the one a large call takes where kernel 3 with the
-                                  automatic number of walkers does not fit */
+                                  automatic number of walkers does not fit or is the slower one */
     LAP_STAT_FALLBACKS = 3,    /* samples re-run with kernel 1 after kernel 2 or 3 withdrew them, since
                                   lap_set_root (synchronises) */
     LAP_STAT_LAST_KERNEL = 4,  /* kernel of the last lap_sample call (0 before any) */

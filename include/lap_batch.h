@@ -35,8 +35,10 @@ typedef struct lap_batch lap_batch;
 /* Options for lap_batch_set_option.  While LANES, CLAIM, BLOCK and STACK have their
  * defaults (or LANES and CLAIM those of lap_batch_autotune) and PATHS is 0, a run
  * samples every graph with the kernels of single graphs on parallel branches, as far
- * as the workspace holds them, and these options describe the persistent sampler
- * that takes the other graphs and runs.  Counts are the same. */
+ * as the workspace holds them and unless the persistent sampler is the faster one for the
+ * batch by an estimate (many small graphs, many samples of small graphs), and these
+ * options describe the persistent sampler that takes the other graphs and runs.  Counts
+ * are the same. */
 typedef enum {
     LAP_BOPT_LANES = 1,  /* samples in flight (one per GPU thread); 0 = as many as the workspace
                             and the resident-thread capacity allow */
